@@ -441,6 +441,7 @@ __global__ void __launch_bounds__(kBlock, 2) cocg_block(BlockArgs<R> a) {
                 a.r[o] = rn;
                 acc_rr(acc[0], acc[1], acc[2], rn);
             }
+            end_rr(acc[0], acc[1], acc[2]);
             block_cols<T, 3, kNvB>(acc, s.scratch, a.partB, G, cta);
             block_cols<T, 1, kNvB>(nb, s.scratch, a.partB, G, cta, 3);
         }

@@ -3,6 +3,7 @@
 // deterministic block / grid reductions used by the persistent solver kernels.
 #pragma once
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include "scocg.h"
@@ -23,26 +24,36 @@ __host__ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
 __host__ __device__ __forceinline__ double2 cscale(double2 a, double s) { return c2(a.x * s, a.y * s); }
 __host__ __device__ __forceinline__ double cabs2(double2 a) { return a.x * a.x + a.y * a.y; }
 __host__ __device__ __forceinline__ double cabs_(double2 a) { return hypot(a.x, a.y); }
-// a / b with scaling by the larger component of b (Smith's method) so that
-// |b| near the limits of the exponent range neither overflows nor underflows.
+// 2^-e / |bs|^2 for bs = 2^-e b, e the exponent of b's larger component (so
+// |bs|^2 lies in [1, 8) and neither overflows nor underflows).
+__host__ __device__ __forceinline__ double scaled_recip(double2 b, double2& bs) {
+#ifdef __CUDA_ARCH__
+    const int e = max(__double2hiint(b.x) & 0x7ff00000, __double2hiint(b.y) & 0x7ff00000) >> 20;
+    const double s = __hiloint2double((2046 - min(e, 2045)) << 20, 0);
+    bs = c2(b.x * s, b.y * s);
+    return __drcp_rn(fma(bs.x, bs.x, bs.y * bs.y)) * s;
+#else
+    int e = 0;
+    frexp(fmax(fabs(b.x), fabs(b.y)), &e);
+    const double s = ldexp(1.0, e < 1022 ? -e : -1022);
+    bs = c2(b.x * s, b.y * s);
+    return 1.0 / (bs.x * bs.x + bs.y * bs.y) * s;
+#endif
+}
+// a / b = a conj(b) / |b|^2.  One reciprocal instead of the two dependent
+// divisions of Smith's method: these quotients (alpha, beta) sit on the serial
+// path of every seed iteration, and an FP64 division is a ~580-cycle chain on
+// this GPU (a reciprocal ~390, a dependent FMA 65).
 __host__ __device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
-    if (fabs(b.x) >= fabs(b.y)) {
-        const double r = b.y / b.x, inv = 1.0 / (b.x + b.y * r);
-        return c2((a.x + a.y * r) * inv, (a.y - a.x * r) * inv);
-    } else {
-        const double r = b.x / b.y, inv = 1.0 / (b.x * r + b.y);
-        return c2((a.x * r + a.y) * inv, (a.y * r - a.x) * inv);
-    }
+    double2 bs;
+    const double inv = scaled_recip(b, bs);
+    return c2(fma(a.x, bs.x, a.y * bs.y) * inv, fma(a.y, bs.x, -(a.x * bs.y)) * inv);
 }
 // 1 / b with the same scaling
 __host__ __device__ __forceinline__ double2 crecip(double2 b) {
-    if (fabs(b.x) >= fabs(b.y)) {
-        const double r = b.y / b.x, inv = 1.0 / (b.x + b.y * r);
-        return c2(inv, -r * inv);
-    } else {
-        const double r = b.x / b.y, inv = 1.0 / (b.x * r + b.y);
-        return c2(r * inv, -inv);
-    }
+    double2 bs;
+    const double inv = scaled_recip(b, bs);
+    return c2(bs.x * inv, -bs.y * inv);
 }
 __host__ __device__ __forceinline__ bool cfinite(double2 a) { return isfinite(a.x) && isfinite(a.y); }
 
@@ -138,6 +149,9 @@ __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long
     asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
 }
+__device__ __forceinline__ void red_release_u64(unsigned long long* p, unsigned long long v) {
+    asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
 __device__ __forceinline__ int ld_volatile_i32(const int* p) {
     int v;
     asm volatile("ld.volatile.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -166,21 +180,27 @@ __device__ __forceinline__ bool grid_barrier(const GridSync& g, unsigned long lo
     if (threadIdx.x == 0) {
         ++epoch;
         const unsigned long long target = epoch * (unsigned long long)g.nctas;
-        __threadfence();
-        if (!skip_arrival) atomicAdd(g.count, 1ull);
+        // release: the CTA's earlier writes (ordered by the barrier above) are
+        // visible to whoever acquires this arrival
+        if (!skip_arrival) red_release_u64(g.count, 1ull);
         int ok = 1;
-        const uint64_t t0 = globaltimer_ns();
-        while (ld_acquire_u64(g.count) < target) {
+        uint64_t t0 = 0;
+        // only the counter is polled on every turn; the error word and the
+        // clock cost a round trip each and are looked at every 64th turn.  A
+        // barrier whose every CTA has arrived passes; a CTA that has left
+        // arrives at no later one, where the others find the error word set.
+        for (unsigned turn = 1; ld_acquire_u64(g.count) < target; ++turn) {
+            if (turn & 63u) continue;
             if (ld_volatile_i32(g.status) < 0) { ok = 0; break; }
-            if (globaltimer_ns() - t0 > g.timeout_ns) {
+            const uint64_t t = globaltimer_ns();
+            if (t0 == 0) t0 = t;
+            if (t - t0 > g.timeout_ns) {
                 atomicCAS(g.status, 0, (int)SCOCG_ERR_TIMEOUT);
                 atomicCAS(g.status, 1, (int)SCOCG_ERR_TIMEOUT);
                 ok = 0;
                 break;
             }
         }
-        if (ok && ld_volatile_i32(g.status) < 0) ok = 0;
-        __threadfence();   // acquire side: later loads of this CTA see the other CTAs' writes
         s_ok = ok;
     }
     __syncthreads();
@@ -220,67 +240,48 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 
-// Sum `nval` per-thread doubles over the CTA; the result lands in out[0..nval)
-// (shared memory) and is visible to all threads after the call.  `scratch`
-// must hold kWarps * nval doubles.
-__device__ __forceinline__ void block_sum(const double* vals, int nval, double* scratch, double* out) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int j = 0; j < nval; ++j) {
-        double v = warp_sum(vals[j]);
-        if (lane == 0) scratch[warp * nval + j] = v;
+// One lane's share of a sum over G per-CTA values p[c * stride], c = lane,
+// lane + 32, ...: the loads are issued together (one L2 round trip up to 512
+// CTAs) and added as a tree over the groups that exist (an FP64 add is a
+// 65-cycle step and holds the SM's FP64 pipe 16 cycles, so neither a serial
+// chain nor adds of absent values are free).
+__device__ __forceinline__ double lane_share(const double* p, size_t stride, int lane, int G) {
+    double tot = 0.0;
+    for (int c0 = 0; c0 < G; c0 += 32 * 16) {
+        double v[16];
+        const int m = min(16, (G - c0 + 31) >> 5);    // groups of 32 values
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+            const int c = c0 + lane + 32 * u;
+            v[u] = c < G ? __ldcg(p + (size_t)c * stride) : 0.0;
+        }
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+            for (int u = 0; u < o; ++u)
+                if (u + o < m) v[u] += v[u + o];
+        tot = c0 == 0 ? v[0] : tot + v[0];
     }
-    __syncthreads();
-    for (int j = threadIdx.x; j < nval; j += blockDim.x) {
-        double s = 0.0;
-        for (int w = 0; w < kWarps; ++w) s += scratch[w * nval + j];
-        out[j] = s;
-    }
-    __syncthreads();
+    return tot;
 }
 
-// Deterministic grid reduction of per-CTA partials part[cta * stride + j],
-// j < nval: every CTA computes bit-identical sums (same data, same order).
-// The loads of a lane are issued together (up to 16 per lane, grids up to 512
-// CTAs in one round) so that the reduction costs one L2 round trip.
-// The same sum over value-major partials part[j * G + cta]: a warp's load of
-// 32 consecutive CTAs is one coalesced request, and the CTAs' reads after a
-// barrier touch G / 32 lines per value instead of G.  Same summation order.
+// Deterministic grid reduction of value-major partials part[j * G + cta]: a
+// warp's load of 32 consecutive CTAs is one coalesced request, and every CTA
+// computes bit-identical sums (same data, same order).
 __device__ __forceinline__ void grid_sum_vm1(const double* part, int nval, double* out, int G) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int j = warp; j < nval; j += kWarps) {
-        const double* pj = part + (size_t)j * G;
-        double s = 0.0;
-        for (int c0 = 0; c0 < G; c0 += 32 * 16) {
-            double v[16];
-#pragma unroll
-            for (int u = 0; u < 16; ++u) {
-                const int c = c0 + lane + 32 * u;
-                v[u] = c < G ? __ldcg(pj + c) : 0.0;
-            }
-#pragma unroll
-            for (int u = 0; u < 16; ++u) s += v[u];
-        }
-        s = warp_sum(s);
+        const double s = warp_sum(lane_share(part + (size_t)j * G, 1, lane, G));
         if (lane == 0) out[j] = s;
     }
     __syncthreads();
 }
 
+// The same over CTA-major partials part[cta * stride + j].
 __device__ __forceinline__ void grid_sum(const double* part, int stride, int nval, double* out, int G) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int j = warp; j < nval; j += kWarps) {
-        double s = 0.0;
-        for (int c0 = 0; c0 < G; c0 += 32 * 16) {
-            double v[16];
-#pragma unroll
-            for (int u = 0; u < 16; ++u) {
-                const int c = c0 + lane + 32 * u;
-                v[u] = c < G ? __ldcg(part + (size_t)c * stride + j) : 0.0;
-            }
-#pragma unroll
-            for (int u = 0; u < 16; ++u) s += v[u];
-        }
-        s = warp_sum(s);
+        const double s = warp_sum(lane_share(part + j, (size_t)stride, lane, G));
         if (lane == 0) out[j] = s;
     }
     __syncthreads();

@@ -56,7 +56,7 @@ struct ResumeState {       // device, written by CTA 0
     int rotated;           // the stopping apply visited its units in the rotated order
     int pad;
     double2 alpha_prev, beta_prev, rho, rho_prev, zs;
-    double rnorm, bnorm;
+    double reserved, bnorm;
     double2 cr_cur[kMaxProj];
 };
 
@@ -96,6 +96,15 @@ __device__ __forceinline__ void load4(const double2* p, double2 (&x)[4]) {
 }
 __device__ __forceinline__ void load4(const float4* p, float4 (&x)[4]) {
     x[0] = p[0]; x[1] = p[1]; x[2] = p[2]; x[3] = p[3];
+}
+
+// z x - a (a: an apply's accumulator)
+__device__ __forceinline__ float2 zx_minus(float2 z, float2 x, float2 a) { return vsub(vcfma(z, x, vzero<float2>()), a); }
+__device__ __forceinline__ double2 zx_minus(double2 z, double2 x, double2 a) {
+    return vcfma(z, x, make_double2(-a.x, -a.y));
+}
+__device__ __forceinline__ float4 zx_minus(float4 z, float4 x, float4 a) {
+    return vcfma(z, x, make_float4(-a.x, -a.y, -a.z, -a.w));
 }
 
 // acc += the accumulator of the lane at distance o (xor), for the row sums
@@ -145,7 +154,7 @@ struct ApplyCSR {
 #pragma unroll
         for (int o = LPR / 2; o > 0; o >>= 1) lane_add(acc, o);
         if (row < n && l == 0) {
-            w = vsub(vcfma(zs, x[row], vzero<VV>()), acc);
+            w = zx_minus(zs, x[row], acc);
             return true;
         }
         return false;
@@ -217,7 +226,7 @@ struct ApplyBSR4 {
             for (int j = 0; j < kG; ++j) block_fma(acc, cb[j], v[j], x);
         }
         if (row < n) {
-            w = vsub(vcfma(zs, x[row], vzero<VV>()), acc);
+            w = zx_minus(zs, x[row], acc);
             return true;
         }
         return false;
@@ -300,7 +309,7 @@ struct ApplyBSR4C {
         VV mine = b0 ? k1 : k0;
         mine.x += t.x; mine.y += t.y;
         if (row < n) {
-            w = vsub(vcfma(zs, x[row], vzero<VV>()), mine);
+            w = zx_minus(zs, x[row], mine);
             return true;
         }
         return false;
@@ -376,9 +385,8 @@ constexpr int kScratch = kWarps * (3 + 2 * kMaxProj) > kScratchNV * kBlock ? kWa
 struct SeedScalars {
     double2 alpha, alpha_prev, beta_prev, rho, rho_prev, zs;
     double2 t2;                 // alpha_n beta_{n-1} / alpha_{n-1}
-    double rnorm, bnorm, rn_b;  // rn_b = ||r_{n+1}|| / ||b||
+    double bnorm, inv_b2;       // ||b||, 1 / ||b||^2
     double2 beta_next;          // rho_{n+1} / rho_n, before it becomes beta_prev
-    double rnorm_next;          // ||r_{n+1}||, before it becomes rnorm
     int seed, active, n;
     int replace_on, n_switch, n_replace;
     long long shift_iters;
@@ -387,16 +395,5 @@ struct SeedScalars {
     double red[4 + 2 * kMaxProj + 4];
     double scratch[kScratch];
 };
-
-// residual estimate of a shift from the seed residual norm and its pi
-__device__ __forceinline__ double shift_resid(double rnorm, double2 pi, double bnorm) {
-    return rnorm / (cabs_(pi) * bnorm);
-}
-
-// Fixed-order complex dot contribution c^T r in FP64
-__device__ __forceinline__ void acc_dot(double2& s, double2 a, double2 b) {
-    s.x = fma(a.x, b.x, fma(-a.y, b.y, s.x));
-    s.y = fma(a.x, b.y, fma(a.y, b.x, s.y));
-}
 
 }  // namespace scocg

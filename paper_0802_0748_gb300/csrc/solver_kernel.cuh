@@ -8,9 +8,8 @@
 namespace scocg {
 
 // A warp sum parked in a double-sized scratch slot in its own type, so that
-// only the final sum over warps (NV threads of warp 0) uses the FP64 pipe:
-// on this GPU an FP64 instruction issued by every warp of an SM holds the
-// FP64 pipe for hundreds of cycles.
+// only the final sum over warps uses the FP64 pipe: an FP64 instruction holds
+// the SM's FP64 pipe for 16 cycles whatever its active lanes.
 __device__ __forceinline__ void park(double* slot, double v) { *slot = v; }
 __device__ __forceinline__ void park(double* slot, float v) { *reinterpret_cast<float*>(slot) = v; }
 __device__ __forceinline__ void park(double* slot, dfs v) { *reinterpret_cast<dfs*>(slot) = v; }
@@ -23,40 +22,54 @@ template <> __device__ __forceinline__ double unpark<dfs>(const double* slot) {
     return to_double(*reinterpret_cast<const dfs*>(slot));
 }
 
-// CTA sum of per-thread values: the warp-level part in the values' own type
-// (FP32 for complex64 vectors), the sum over warps in FP64.
+// CTA sums of the first nv of NV per-thread values, of which only the warps
+// with place wi < nw hold any: warp j < nv writes sum j to part[j * G] (the caller
+// synchronises the CTA before anyone reads it or reuses scratch).  Each sum is
+// a tree, not a chain: a serial FP64 chain over 16 warps was ~0.5 us of every
+// seed iteration, twice.
 template <int NV, typename T>
-__device__ __forceinline__ void block_sum_n(T (&v)[NV], double* scratch, double* out) {
+__device__ __forceinline__ void block_partials(T (&v)[NV], double* scratch, double* part, int G, int wi,
+                                               int nv = NV, int nw = kWarps) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if constexpr (std::is_same<T, double>::value) {
         // FP64 values: every thread parks its values (scratch holds NV *
-        // kBlock doubles) and NV warps sum them, instead of NV five-step FP64
-        // warp sums in all kWarps warps (an FP64 instruction of a whole warp
-        // occupies the FP64 pipe ~16 cycles)
+        // kBlock doubles) and nv warps sum them, instead of five-step FP64
+        // warp sums in all warps
         static_assert(NV <= kScratchNV, "scratch too small");
+        if (wi < nw)
 #pragma unroll
-        for (int j = 0; j < NV; ++j) scratch[j * kBlock + threadIdx.x] = v[j];
+            for (int j = 0; j < NV; ++j)
+                if (j < nv) scratch[j * kBlock + 32 * wi + lane] = v[j];
         __syncthreads();
-        if (warp < NV) {
-            double acc = 0.0;
-            for (int t = lane; t < kBlock; t += 32) acc += scratch[warp * kBlock + t];
-            acc = warp_sum(acc);
-            if (lane == 0) out[warp] = acc;
+        if (warp < nv) {
+            double a[4] = {0.0, 0.0, 0.0, 0.0};
+            for (int w = 0; w < nw; w += 4)
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (w + q < nw) {
+                        const double t = scratch[warp * kBlock + 32 * (w + q) + lane];
+                        a[q] = w == 0 ? t : a[q] + t;
+                    }
+            if (nw > 2) { a[0] += a[2]; if (nw > 3) a[1] += a[3]; }
+            if (nw > 1) a[0] += a[1];
+            const double t = warp_sum(a[0]);
+            if (lane == 0) part[(size_t)warp * G] = t;
         }
-        __syncthreads();
     } else {
+        // the warp-level part in the values' own type, the sum over warps in FP64
 #pragma unroll
         for (int j = 0; j < NV; ++j) {
+            if (j >= nv) break;
             const T t = warp_sum(v[j]);
-            if (lane == 0) park(scratch + warp * NV + j, t);
+            if (lane == 0) park(scratch + j * kWarps + wi, t);
         }
         __syncthreads();
-        if (threadIdx.x < NV) {
-            double s = 0.0;
-            for (int w = 0; w < kWarps; ++w) s += unpark<T>(scratch + w * NV + threadIdx.x);
-            out[threadIdx.x] = s;
+        if (warp < nv) {
+            double t = lane < kWarps ? unpark<T>(scratch + warp * kWarps + lane) : 0.0;
+#pragma unroll
+            for (int o = kWarps / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (lane == 0) part[(size_t)warp * G] = t;
         }
-        __syncthreads();
     }
 }
 
@@ -84,11 +97,27 @@ __device__ __forceinline__ void acc_nrm(dfs& s, float4 u) {
     df_acc_prod(s, cim(u), cim(u));
 }
 
-// Per-thread accumulation of rho = r^T r (re, im) and ||r||^2.
+// Per-thread accumulation of rho = r^T r and ||r||^2, and the thread's totals
+// (re rho, im rho, ||r||^2) after its last row.
 template <typename AT, typename V>
 __device__ __forceinline__ void acc_rr(AT& re, AT& im, AT& nrm, V ri) {
     acc_bil(re, im, ri, ri);
     acc_nrm(nrm, ri);
+}
+template <typename AT>
+__device__ __forceinline__ void end_rr(AT&, AT&, AT&) {}
+// complex128: sum of x^2 - y^2, of x y and of y^2 (four FP64 FMAs a row
+// instead of six), combined once per thread
+template <>
+__device__ __forceinline__ void acc_rr<double, double2>(double& re, double& xy, double& yy, double2 ri) {
+    re = fma(ri.x, ri.x, fma(-ri.y, ri.y, re));
+    xy = fma(ri.x, ri.y, xy);
+    yy = fma(ri.y, ri.y, yy);
+}
+template <>
+__device__ __forceinline__ void end_rr<double>(double& re, double& xy, double& yy) {
+    xy += xy;
+    yy = fma(2.0, yy, re);
 }
 // Compensated vectors: rho = sum (x^2 - y^2) + 2i sum x y from three
 // pair-exact products (the doubling is exact), and ||r||^2 from the high
@@ -119,37 +148,41 @@ __device__ __forceinline__ void acc_r(typename Acc<R>::T (&acc)[5], typename Vec
 template <typename V>
 __device__ __forceinline__ V r_update(V r, V al, V q) { return vsub(r, vcfma(al, q, vzero<V>())); }
 template <>
+__device__ __forceinline__ double2 r_update<double2>(double2 r, double2 al, double2 q) {
+    return vcfma(make_double2(-al.x, -al.y), q, r);
+}
+template <>
 __device__ __forceinline__ float4 r_update<float4>(float4 r, float4 al, float4 q) {
     return vcfma(make_float4(-al.x, -al.y, -al.z, -al.w), q, r);
 }
 
-// CTA sum of the accumulated partials into values 0..4 of this CTA's column
-// of the value-major partials (value j at part[j * G]); the extra dense
-// projections m >= 1 are summed in separate passes over r into values 3 + 2m.
+// CTA sums of the accumulated partials into values 0..2 (0..4 with dense
+// projections) of this CTA's column of the value-major partials (value j at
+// part[j * G]); the extra dense projections m >= 1 are summed in separate
+// passes over r into values 3 + 2m.
 template <typename R>
-__device__ __forceinline__ void finish_r_partials(const SolveArgs<R>& a, const typename Acc<R>::T (&acc)[5],
-                                                  int64_t rbeg, int64_t rend, SeedScalars& s, double* s_part,
-                                                  double* part, int G) {
+__device__ __forceinline__ void finish_r_partials(const SolveArgs<R>& a, typename Acc<R>::T (&acc)[5],
+                                                  int64_t rbeg, int64_t rend, SeedScalars& s, double* part, int G) {
     using AT = typename Acc<R>::T;
     const int tid = threadIdx.x;
-    AT v[5] = {acc[0], acc[1], acc[2], acc[3], acc[4]};
-    block_sum_n<5>(v, s.scratch, s_part);
-    if (tid < 5) part[(size_t)tid * G] = s_part[tid];
+    const int nw = (int)min((int64_t)kWarps, (rend - rbeg + 31) >> 5);   // warps that hold rows
+    end_rr(acc[0], acc[1], acc[2]);
+    block_partials<5>(acc, s.scratch, part, G, tid >> 5, a.cvec ? 5 : 3, max(nw, 1));
     for (int m = 1; m < a.nproj && a.cvec; ++m) {
         AT w2[2] = {};
         for (int64_t i = rbeg + tid; i < rend; i += kBlock) acc_bil(w2[0], w2[1], a.cvec[(size_t)m * a.n + i], a.r[i]);
-        block_sum_n<2>(w2, s.scratch, s_part);
-        if (tid < 2) part[(size_t)(3 + 2 * m + tid) * G] = s_part[tid];
+        __syncthreads();   // the sums above have been read from scratch
+        block_partials<2>(w2, s.scratch, part + (size_t)(3 + 2 * m) * G, G, tid >> 5, 2, max(nw, 1));
     }
 }
 
 template <typename R>
 __device__ __forceinline__ void r_partials(const SolveArgs<R>& a, int64_t rbeg, int64_t rend,
-                                           SeedScalars& s, double* s_part, double* part, int G) {
+                                           SeedScalars& s, double* part, int G) {
     typename Acc<R>::T acc[5] = {};
     for (int64_t i = rbeg + threadIdx.x; i < rend; i += kBlock)
         acc_r<R>(acc, a.r[i], a.cvec ? a.cvec + i : nullptr);
-    finish_r_partials(a, acc, rbeg, rend, s, s_part, part, G);
+    finish_r_partials(a, acc, rbeg, rend, s, part, G);
 }
 
 #ifdef SCOCG_CHECKED
@@ -236,14 +269,29 @@ struct HasTwoPass<A, std::void_t<decltype(A::kTwoPass)>> : std::integral_constan
 // ends the solve with that status (SCOCG_OK is 0, so 0 cannot mean "go on").
 constexpr int kGoOn = 0x7fffffff;
 
+// Phase A's third partial: the unconverged shifts of a CTA after the last
+// phase C and whether a pi^k became zero or non-finite, as two integers (their
+// sums need no FP64 arithmetic).
+__device__ __forceinline__ double pack_counts(int active, int bad) { return __hiloint2double(bad, active); }
+__device__ __forceinline__ void sum_counts(const double* part, int G, int& active, int& bad) {
+    const int lane = threadIdx.x & 31;
+    int act = 0, any = 0;
+    for (int c = lane; c < G; c += 32) {
+        const double v = __ldcg(part + c);
+        act += __double2loint(v);
+        any |= __double2hiint(v);
+    }
+    active = __reduce_add_sync(0xffffffffu, act);
+    bad = __reduce_or_sync(0xffffffffu, any);
+}
+
 // The first phase A of a solve continued from a ResumeState: the stopped
 // apply's r^T q partial again, from the stored r_n and q_n over the same rows
 // in the same order (so the continued solve matches an uninterrupted one bit
 // for bit), and the shift count as its deferred phase C left it.
 template <typename R, class Apply>
 __device__ __forceinline__ void resume_partials(const SolveArgs<R>& a, const Apply& ap, int G, int cta, int64_t ubeg,
-                                             int64_t u_end, int64_t u_step, bool active, SeedScalars& s,
-                                             double* s_part) {
+                                             int64_t u_end, int64_t u_step, int nwA, bool active, SeedScalars& s) {
     using AT = typename Acc<R>::T;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool rot = a.rstate->rotated != 0;
@@ -255,13 +303,8 @@ __device__ __forceinline__ void resume_partials(const SolveArgs<R>& a, const App
         if (ap.row_of(u, lane, row)) acc_bil(rq[0], rq[1], a.r[row], a.q[row]);
     }
     const int act = __syncthreads_count(active);
-    block_sum_n<2>(rq, s.scratch, s_part);
-    if (tid == 0) {
-        double* pa = a.partA + cta;
-        pa[0] = s_part[0]; pa[G] = s_part[1];
-        pa[2 * G] = (double)act;
-        pa[3 * G] = 0.0;
-    }
+    block_partials<2>(rq, s.scratch, a.partA + cta, G, wi, 2, nwA);
+    if (tid == 64) a.partA[2 * G + cta] = pack_counts(act, 0);
     __syncthreads();
 }
 
@@ -275,7 +318,7 @@ static __device__ __noinline__ void save_resume_state(ResumeState* rs, const See
     rs->replace_on = s.replace_on;
     rs->rotated = rotated;
     rs->alpha_prev = s.alpha_prev; rs->beta_prev = s.beta_prev; rs->rho = s.rho; rs->rho_prev = s.rho_prev;
-    rs->zs = s.zs; rs->rnorm = s.rnorm; rs->bnorm = s.bnorm;
+    rs->zs = s.zs; rs->reserved = 0.0; rs->bnorm = s.bnorm;
     for (int m = 0; m < M; ++m) rs->cr_cur[m] = s.cr_cur[m];
 }
 
@@ -291,8 +334,7 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
     constexpr bool kMixed = std::is_same<R, float>::value;   // complex64 vectors
     constexpr bool kFull = std::is_same<R, double>::value;   // full-vector mode compiled (FP64 only)
     __shared__ SeedScalars s;
-    __shared__ double s_part[8];
-    __shared__ int s_flag[5];
+    __shared__ int s_flag[7];            // 0, 1: this CTA's shift counts; 2, 3: decision; 4: seed converged; 5, 6: grid counts
     __shared__ double s_min[kWarps];
     __shared__ int s_arg[kWarps];
     __shared__ ShiftInputs s_c;          // inputs of a deferred phase C
@@ -311,6 +353,10 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
     const int64_t u_first = Apply::kMap == kMapStrided ? (int64_t)cta + (int64_t)G * warp : ubeg + warp;
     const int64_t u_step = kWhole ? (int64_t)G * kWarps : kWarps;
     const int64_t u_end = kWhole ? a.nunits : uend;
+    // warps that visit a unit (all of them when there are enough)
+    const int64_t u_cnt = Apply::kMap == kMapStrided ? (a.nunits - cta + G - 1) / G
+                          : kWhole ? a.nunits : uend - ubeg;
+    const int nwA = (int)max((int64_t)1, min((int64_t)kWarps, u_cnt));
     const int64_t rbeg = (int64_t)cta * a.n / G, rend = (int64_t)(cta + 1) * a.n / G;
     const int M = a.nproj;
     const bool dense_proj = a.cvec != nullptr;
@@ -342,7 +388,7 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
             const ResumeState& rs = *a.rstate;
             s.rho = rs.rho; s.rho_prev = rs.rho_prev;
             s.alpha_prev = rs.alpha_prev; s.beta_prev = rs.beta_prev;
-            s.bnorm = rs.bnorm; s.rnorm = rs.rnorm;
+            s.bnorm = rs.bnorm; s.inv_b2 = 1.0 / (s.bnorm * s.bnorm);
             s.seed = rs.seed; s.zs = rs.zs;
             s_vs[0] = Vec<R>::make(s.zs);
             s_vs[1] = Vec<R>::make(s.beta_prev);
@@ -357,7 +403,7 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
         // that a stop right after this pass records the stopped one's order
         if (tid < 5) s_flag[tid] = tid == 4 ? (a.rstate->rotated ? 0 : 1) : 0;
         __syncthreads();
-        resume_partials(a, ap, G, cta, ubeg, u_end, u_step, owns && !a.S.frozen[k_own], s, s_part);
+        resume_partials(a, ap, G, cta, ubeg, u_end, u_step, nwA, owns && !a.S.frozen[k_own], s);
     } else {
         double nb = 0.0;
         for (int64_t i = rbeg + tid; i < rend; i += kBlock) {
@@ -373,10 +419,9 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
             nb = fma(bi.x, bi.x, fma(bi.y, bi.y, nb));
         }
         double v1[1] = {nb};
-        block_sum_n<1>(v1, s.scratch, s_part);
-        if (tid == 0) a.partC[(size_t)cta * kPartC] = s_part[0];
+        block_partials<1>(v1, s.scratch, a.partC + (size_t)cta * kPartC, G, warp);
         __syncthreads();
-        r_partials(a, rbeg, rend, s, s_part, myB, G);
+        r_partials(a, rbeg, rend, s, myB, G);
         if (owns) {
             const int k = k_own;
             a.S.pi_prev[k] = c2(1, 0); a.S.pi_cur[k] = c2(1, 0); a.S.inv_cur[k] = c2(1, 0);
@@ -385,14 +430,14 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
             for (int m = 0; m < M; ++m) { a.S.P[(size_t)k * M + m] = c2(0, 0); a.S.X[(size_t)k * M + m] = c2(0, 0); }
             a.S.frozen[k] = 0; a.S.iters[k] = 0; a.S.resid[k] = 1.0;
         }
-        if (tid < 5) s_flag[tid] = 0;
+        if (tid < 7) s_flag[tid] = 0;
         if (!grid_barrier(a.sync, epoch)) return;
         grid_sum_vm1(a.partB, nred, s.red, G);
         grid_sum(a.partC, kPartC, 1, s.red + nred, G);
         if (tid == 0) {
             s.rho = c2(s.red[0], s.red[1]);
             s.bnorm = sqrt(s.red[nred]);
-            s.rnorm = s.bnorm;
+            s.inv_b2 = 1.0 / (s.bnorm * s.bnorm);
             s.alpha_prev = c2(1, 0);
             s.beta_prev = c2(0, 0);
             s.seed = a.seed;
@@ -460,14 +505,9 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
                     }
                 }
             }
-            block_sum_n<2>(rq, s.scratch, s_part);
+            block_partials<2>(rq, s.scratch, a.partA + cta, G, wi, 2, nwA);
             pending = false;
-            if (tid == 0) {
-                double* pa = a.partA + cta;            // value-major
-                pa[0] = s_part[0]; pa[G] = s_part[1];
-                pa[2 * G] = (double)s_flag[0];   // unconverged shifts of this CTA after the last phase C
-                pa[3 * G] = (double)s_flag[1];   // a pi^k of this CTA became zero or non-finite
-            }
+            if (tid == 64) a.partA[2 * G + cta] = pack_counts(s_flag[0], s_flag[1]);
         }
         skip_a = false;
         SCOCG_TRACE(2);
@@ -475,12 +515,17 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
         if (!grid_barrier(a.sync, epoch, a.debug_inject == 1 && cta == 0 && s.n == 3)) return;
         SCOCG_TRACE(3);
         SCOCG_MARK(1);
-        grid_sum_vm1(a.partA, 4, s.red, G);
+        if (warp == 2) {
+            int act, bad;
+            sum_counts(a.partA + 2 * G, G, act, bad);
+            if (lane == 0) { s_flag[5] = act; s_flag[6] = bad; }
+        }
+        grid_sum_vm1(a.partA, 2, s.red, G);
         if (tid == 0) {
             const double2 rq = c2(s.red[0], s.red[1]);
-            const int active = s.n == 0 ? a.K : (int)s.red[2];
+            const int active = s.n == 0 ? a.K : s_flag[5];
             int st = kGoOn;
-            if (s.n > 0 && s.red[3] != 0.0) st = SCOCG_ERR_BREAKDOWN;
+            if (s.n > 0 && s_flag[6] != 0) st = SCOCG_ERR_BREAKDOWN;
             else if (active == 0) st = SCOCG_OK;
             else if (s.n >= a.max_iter) st = SCOCG_NOT_CONVERGED;
             else if (cabs2(s.rho) == 0.0 || cabs2(rq) == 0.0 || !cfinite(rq)) st = SCOCG_ERR_BREAKDOWN;
@@ -588,7 +633,7 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
                 acc_r<R>(acc, rn, a.cvec ? a.cvec + i : nullptr);
             }
             __syncthreads();
-            finish_r_partials(a, acc, rbeg, rend, s, s_part, myB, G);
+            finish_r_partials(a, acc, rbeg, rend, s, myB, G);
         }
         SCOCG_TRACE(4);
         SCOCG_MARK(2);
@@ -597,8 +642,8 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
         SCOCG_MARK(3);
         grid_sum_vm1(a.partB, nred, s.red, G);
         SCOCG_MARK(5);
-        // the scalars of this iteration: independent FP64 divisions and roots
-        // run in three warps at once
+        // the scalars of this iteration: independent FP64 chains run in three
+        // warps at once
         if (tid < M) {
             s.cr_next[tid] = dense_proj ? c2(s.red[3 + 2 * tid], s.red[4 + 2 * tid])
                                         : (chk(a.dbg, 12, a.cidx[tid], a.n) ? Vec<R>::wide(__ldcg(a.r + a.cidx[tid])) : c2(0, 0));
@@ -608,9 +653,7 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
             s.t2 = cdiv(cmul(s.alpha, s.beta_prev), s.alpha_prev);
             s_c.alpha = s.alpha; s_c.beta_prev = s.beta_prev; s_c.t2 = s.t2; s_c.n = s.n;
         } else if (tid == 32) {
-            s.rnorm_next = sqrt(s.red[2]);
-            s.rn_b = s.rnorm_next / s.bnorm;
-            s_c.rn_b2 = s.rn_b * s.rn_b;
+            s_c.rn_b2 = s.red[2] * s.inv_b2;
             s_flag[4] = a.tol > 0.0 && s_c.rn_b2 <= tol2;    // the seed (pi = 1) has converged
         } else if (tid == 64) {
             s.beta_next = cdiv(c2(s.red[0], s.red[1]), s.rho);
@@ -636,7 +679,6 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
             s.alpha_prev = s.alpha;
             s.rho_prev = s.rho;
             s.rho = c2(s.red[0], s.red[1]);
-            s.rnorm = s.rnorm_next;
             s.n += 1;
         }
         if (tid < M) s.cr_cur[tid] = s.cr_next[tid];
@@ -731,7 +773,6 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
                 s.rho = cdiv(s.rho, cmul(pin1, pin1));
                 s.beta_prev = cmul(cmul(ratio, ratio), s.beta_prev);
                 s.alpha_prev = alpha_s2;
-                s.rnorm = s.rnorm / cabs_(pin1);
                 s.seed = s2;
                 s.zs = a.z[s2];
                 s_vs[0] = Vec<R>::make(s.zs);
@@ -763,14 +804,13 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
                     }
                 }
                 if (!grid_barrier(a.sync, epoch)) return;
-                r_partials(a, rbeg, rend, s, s_part, myB, G);
+                r_partials(a, rbeg, rend, s, myB, G);
                 if (!grid_barrier(a.sync, epoch)) return;
                 grid_sum_vm1(a.partB, nred, s.red, G);
                 if (tid == 0) {
                     s.rho = c2(s.red[0], s.red[1]);
                     s.beta_prev = cdiv(s.rho, s.rho_prev);
                     s_vs[1] = Vec<R>::make(s.beta_prev);
-                    s.rnorm = sqrt(s.red[2]);
                     s.n_replace += 1;
                 }
                 if (tid < M) {
