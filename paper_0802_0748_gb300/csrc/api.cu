@@ -562,6 +562,10 @@ int scocg::solve_impl(scocg_ctx* h, const scocg_c128* shifts, int nshift, const 
     // chain: 24.4 us per iteration at 8 CTAs, 21.1 at 32)
     int64_t want = std::max<int64_t>((nunits + kWarps - 1) / kWarps, (K + kBlock - 1) / kBlock);
     want = std::max<int64_t>(want, std::min<int64_t>(32, nunits));
+    // full-vector mode: two FP64 vectors per shift are updated every iteration,
+    // so the rows are spread over as many SMs as there are units (16^3 x 4, 64
+    // shifts: 32 CTAs took 80 us per iteration)
+    if (Xf) want = std::max<int64_t>(want, nunits);
     if (h->opts.grid > 0) want = h->opts.grid;
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, maxco));
     if ((int64_t)grid * kBlock < K) return SCOCG_ERR_INVALID;

@@ -374,7 +374,7 @@ struct SolveArgs {
     ResumeState* rstate;
     int resume;
 };
-constexpr int kFullSmem = 3 * 16 + 4;   // per shift: 1/pi_n, beta^k, alpha^k, active flag
+constexpr int kFullSmem = 3 * 16 + 4;   // per shift: two coefficients, the scale of its direction, a list entry
 
 // Shared per-CTA copy of the seed scalars; every CTA holds identical values.
 // CTA scratch of the block sums: per warp 3 + 2 kMaxProj values, or (FP64

@@ -343,6 +343,7 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
     // warps on the FP64 pipe at each phase start)
     __shared__ V s_vs[3];
     SCOCG_DYN_SHARED(double2, s_full);   // full-vector mode: per-shift scalars of the iteration
+    __shared__ int s_nact;               // and the number of unconverged shifts
 
     const int tid = threadIdx.x;
     const int lane = tid & 31, warp = tid >> 5;
@@ -544,31 +545,63 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
         if (s_flag[2] != kGoOn) { status = s_flag[2]; break; }
 
         // ---- full-vector mode: this iteration's shift scalars for all shifts
-        // (every CTA computes them, with the same arithmetic as phase C)
+        // (every CTA computes them, with the same arithmetic as phase C).  The
+        // directions are stored as pt^k = p^k / t_k with t_k = 1 / pi^k of the
+        // iteration that wrote them, so that pt^k_n = r_n + cp pt^k_{n-1} and
+        // x^k += cx pt^k take one complex FMA each:
+        // cp = beta^k t_k pi^k_n, cx = alpha^k / pi^k_n.
         if constexpr (kFull) {
             if (a.Xf) {
-                double2* s_inv = s_full;
-                double2* s_bet = s_full + a.K;
-                double2* s_alp = s_full + 2 * a.K;
-                int* s_act = reinterpret_cast<int*>(s_full + 3 * a.K);
+                double2* s_cp = s_full;
+                double2* s_cx = s_full + a.K;
+                double2* s_t = s_full + 2 * a.K;
+                int* s_list = reinterpret_cast<int*>(s_full + 3 * a.K);   // the unconverged shifts, in any order
+                if (tid == 0) s_nact = 0;
+                __syncthreads();
                 const double2 t2 = cdiv(cmul(s.alpha, s.beta_prev), s.alpha_prev);
                 for (int k = tid; k < a.K; k += kBlock) {
-                    int act = 0;
-                    if (!__ldcg(a.S.frozen + k)) {
-                        const double2 pp = __ldcg(a.S.pi_prev + k), pc = __ldcg(a.S.pi_cur + k);
-                        const double2 ic = __ldcg(a.S.inv_cur + k);
-                        const double2 ratio = cmul(pp, ic);
-                        const double2 pn = cadd(cmul(cadd(c2(1, 0), cmul(s.alpha, __ldcg(a.S.sigma + k))), pc),
-                                                cmul(t2, csub(pc, pp)));
-                        const double2 in = crecip(pn);
-                        s_inv[k] = ic;
-                        s_bet[k] = cmul(cmul(ratio, ratio), s.beta_prev);
-                        s_alp[k] = cmul(cmul(pc, in), s.alpha);
-                        act = 1;
-                    }
-                    s_act[k] = act;
+                    if (__ldcg(a.S.frozen + k)) continue;
+                    const double2 pp = __ldcg(a.S.pi_prev + k), pc = __ldcg(a.S.pi_cur + k);
+                    const double2 ic = __ldcg(a.S.inv_cur + k);
+                    const double2 ratio = cmul(pp, ic);
+                    const double2 pn = cadd(cmul(cadd(c2(1, 0), cmul(s.alpha, __ldcg(a.S.sigma + k))), pc),
+                                            cmul(t2, csub(pc, pp)));
+                    const double2 in = crecip(pn);
+                    const double2 t = s.n == 0 ? c2(1, 0) : s_t[k];
+                    s_cp[k] = cmul(cmul(cmul(cmul(ratio, ratio), s.beta_prev), pc), t);
+                    s_cx[k] = cmul(cmul(cmul(pc, in), s.alpha), ic);
+                    s_t[k] = ic;
+                    s_list[atomicAdd(&s_nact, 1)] = k;
                 }
                 __syncthreads();
+                // Warps take 32-row chunks of the CTA's rows; when there are
+                // fewer chunks than warps, several warps share a chunk's shifts.
+                // Four shifts' vectors are in flight per warp.
+                const int nch = (int)((rend - rbeg + 31) >> 5), nact = s_nact;
+                const int share = nch < kWarps ? kWarps / max(nch, 1) : 1;
+                for (int c = warp / share; c < nch; c += kWarps / share) {
+                    const int64_t i = rbeg + 32 * c + lane;
+                    if (i >= rend) continue;
+                    const double2 ri = a.r[i];
+                    constexpr int kU = 4;
+                    for (int j0 = (warp % share) * kU; j0 < nact; j0 += share * kU) {
+                        double2 p[kU], x[kU];
+                        int kk[kU];
+#pragma unroll
+                        for (int u = 0; u < kU; ++u) {
+                            kk[u] = j0 + u < nact ? s_list[j0 + u] : -1;
+                            if (kk[u] >= 0) { p[u] = a.Pf[(size_t)kk[u] * a.n + i]; x[u] = a.Xf[(size_t)kk[u] * a.n + i]; }
+                        }
+#pragma unroll
+                        for (int u = 0; u < kU; ++u) {
+                            if (kk[u] < 0) continue;
+                            const double2 pn = vcfma(s_cp[kk[u]], p[u], ri);
+                            a.Pf[(size_t)kk[u] * a.n + i] = pn;
+                            a.Xf[(size_t)kk[u] * a.n + i] = vcfma(s_cx[kk[u]], pn, x[u]);
+                        }
+                    }
+                }
+                __syncthreads();   // the rows' r_n have been read
             }
         }
 
@@ -577,8 +610,7 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
             const V al = s_vs[2];
             const V bp = s_vs[1];
             const bool track_x = kMixed && s.replace_on;
-            bool plain = !track_x;
-            if constexpr (kFull) plain = plain && a.Xf == nullptr;
+            const bool plain = !track_x;
             AT acc[5] = {};
             if (plain) {
                 // one row ahead: the next row's loads are in flight while this
@@ -598,20 +630,6 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
             }
             for (int64_t i = rbeg + tid; !plain && i < rend; i += kBlock) {
                 const V ro = a.r[i];
-                if constexpr (kFull) {
-                    if (a.Xf) {
-                        // p^k_n = r_n / pi^k_n + beta^k_{n-1} p^k_{n-1};  x^k_{n+1} = x^k_n + alpha^k_n p^k_n
-                        const int* s_act = reinterpret_cast<const int*>(s_full + 3 * a.K);
-                        const double2 rw = Vec<R>::wide(ro);
-                        for (int k = 0; k < a.K; ++k) {
-                            if (!s_act[k]) continue;
-                            const size_t o = (size_t)k * a.n + i;
-                            const double2 p = vcfma(s_full[a.K + k], a.Pf[o], cmul(rw, s_full[k]));
-                            a.Pf[o] = p;
-                            a.Xf[o] = vcfma(s_full[2 * a.K + k], p, a.Xf[o]);
-                        }
-                    }
-                }
                 if constexpr (kMixed) {
                     if (track_x) {
                         // p_n = r_n + beta_{n-1} p_{n-1};  x_{n+1} = x_n + alpha_n p_n (compensated sum)
