@@ -8,6 +8,7 @@
 #include <cstring>
 #include <new>
 #include <numeric>
+#include <type_traits>
 #include <vector>
 
 #include "api_internal.h"
@@ -124,7 +125,7 @@ int scocg::init_ctx(scocg_ctx* h, const scocg_opts* opts, void* stream) {
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device);
     if (e != cudaSuccess) return cuda_status(e);
     if (!coop) return SCOCG_ERR_CUDA;
-    e = cudaMalloc(&h->d_ctrl, sizeof(Ctrl));
+    e = cudaMalloc((void**)&h->d_ctrl, kCtrlBytes);
     if (e != cudaSuccess) return cuda_status(e);
     h->ws_gen = next_generation();
     h->ws.gen = &h->ws_gen;
@@ -338,10 +339,26 @@ static int solve_one_rhs(scocg_ctx* h, const double2* d_z, int K, int seed, cons
     a.sync.status = &h->d_ctrl->status;
     a.sync.timeout_ns = (uint64_t)(h->opts.timeout_ms * 1e6);
     a.sync.nctas = grid;
+    a.pk = ctrl_packets(h->d_ctrl, grid, cvec != nullptr, M);
     a.stats = &h->d_ctrl->stats;
     a.G = G;
     a.debug_inject = h->opts.debug_inject;
     a.dbg = h->d_ctrl->dbg;
+    // q in shared memory for CSR handles where the grid's SMs can hold it beside
+    // the CTAs that must stay co-resident (22^3 x 4 compensated: 15.4 against
+    // 15.7 us per iteration, 64^3 x 4: 61.2 against 61.3).  Not for the Hubbard
+    // applies: the ring's gathers lose more L1 than q saves (12 sites: 54.6
+    // against 53.1 us), and the two-orbital passes hand q from CTA to CTA.
+    a.q_smem = 0;
+    if (h->kind == HandleKind::kCsr) {
+        const size_t qb = q_smem_bytes<R>(a.nunits, a.rows_per_unit, grid);
+        const int per_sm = (grid + h->num_sms - 1) / h->num_sms;
+        if (qb * per_sm <= kQSmemPerSm) {
+            a.q_smem = 1;
+            const int prec = std::is_same<R, float>::value ? SCOCG_MIXED : std::is_same<R, DF>::value ? SCOCG_MIXED_DF : SCOCG_FP64;
+            a.q_smem = max_coresident_ctas(L, prec, h->num_sms, solve_smem(a, grid)) >= grid;
+        }
+    }
     a.trace = nullptr;
     a.phase_ns = nullptr;
 #ifdef SCOCG_PHASE_TIMERS
@@ -375,7 +392,7 @@ static int solve_one_rhs(scocg_ctx* h, const double2* d_z, int K, int seed, cons
         if (cudaHostGetDevicePointer((void**)&d_trace, g_trace, 0) == cudaSuccess) a.trace = d_trace;
     }
 #endif
-    cudaError_t e = cudaMemsetAsync(h->d_ctrl, 0, sizeof(Ctrl), h->stream);
+    cudaError_t e = cudaMemsetAsync(h->d_ctrl, 0, a.pk ? kCtrlBytes : sizeof(Ctrl), h->stream);
     if (e != cudaSuccess) return cuda_status(e);
     if (h->kind == HandleKind::kHubbard) e = hubbard_launch_solve(a, h->hub, grid, h->stream);
     else e = launch_solve<R>(a, L, grid, h->stream);
@@ -528,7 +545,7 @@ int scocg::solve_impl(scocg_ctx* h, const scocg_c128* shifts, int nshift, const 
             return SCOCG_ERR_INVALID;
     }
     if (!resume) h->rs.ok = false;   // any other solve overwrites the state
-    const size_t dyn_smem = Xf ? (size_t)nshift * kFullSmem : 0;
+    const size_t dyn_smem = full_smem(Xf ? nshift : 0);
     const bool mixed = prec == SCOCG_MIXED;
     const bool dfm = prec == SCOCG_MIXED_DF;
     // several right-hand sides with unit projections: the block kernel

@@ -20,6 +20,15 @@ struct Ctrl {
     unsigned long long dbg[4];   // checked builds: (flag, site, index, limit)
 };
 
+// The control block as allocated: the packets of small grids follow it, and
+// both are zeroed before a solve (kCtrlBytes); only Ctrl is read back.
+constexpr size_t kCtrlHead = (sizeof(Ctrl) + 255) / 256 * 256;
+constexpr size_t kCtrlBytes = kCtrlHead + sizeof(ulonglong2) * kPktVals * kPktCtas;
+inline ulonglong2* ctrl_packets(Ctrl* c, int grid, bool dense, int M) {
+    if (grid > kPktCtas || (dense && M > 1)) return nullptr;
+    return reinterpret_cast<ulonglong2*>(reinterpret_cast<char*>(c) + kCtrlHead);
+}
+
 // Sequential carving of a buffer into 256-byte aligned pieces; with a null
 // base it only measures (every piece returns nullptr, `off` is the total).
 struct Carver {

@@ -152,6 +152,18 @@ __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long
 __device__ __forceinline__ void red_release_u64(unsigned long long* p, unsigned long long v) {
     asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
+__device__ __forceinline__ void fence_acq_rel() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+// a {value, tag} pair, written and read in one piece (16-byte aligned)
+__device__ __forceinline__ void st_packet(ulonglong2* p, double v, unsigned long long tag) {
+    asm volatile("{.reg .b128 t; mov.b128 t, {%1, %2}; st.relaxed.gpu.global.b128 [%0], t;}" ::"l"(p),
+                 "l"(__double_as_longlong(v)), "l"(tag) : "memory");
+}
+__device__ __forceinline__ double ld_packet(const ulonglong2* p, unsigned long long& tag) {
+    long long v;
+    asm volatile("{.reg .b128 t; ld.relaxed.gpu.global.b128 t, [%2]; mov.b128 {%0, %1}, t;}"
+                 : "=l"(v), "=l"(tag) : "l"(p) : "memory");
+    return __longlong_as_double(v);
+}
 __device__ __forceinline__ int ld_volatile_i32(const int* p) {
     int v;
     asm volatile("ld.volatile.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");

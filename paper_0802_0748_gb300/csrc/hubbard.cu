@@ -333,6 +333,12 @@ static ApplyHubbard<R> make_apply(const Hubbard& hb) {
 int hubbard_max_ctas(const Hubbard& hb, int prec, int num_sms, size_t dyn_smem) {
     if (hb.model == 1) return hubbard2_max_ctas(hb, prec, num_sms, dyn_smem);
     int nb = 0;
+    if (dyn_smem > 0) {   // above the 48 KB default together with the static part
+        const void* k = prec == SCOCG_MIXED      ? (const void*)cocg_persistent<float, ApplyHubbard<float>>
+                        : prec == SCOCG_MIXED_DF ? (const void*)cocg_persistent<DF, ApplyHubbard<float>>
+                                                 : (const void*)cocg_persistent<double, ApplyHubbard<double>>;
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemMax);
+    }
     cudaError_t e =
         prec == SCOCG_MIXED
             ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, cocg_persistent<float, ApplyHubbard<float>>, kBlock,
@@ -353,12 +359,12 @@ cudaError_t hubbard_launch_solve(const SolveArgs<R>& a, const Hubbard& hb, int g
     ApplyHubbard<W> ap = make_apply<W>(hb);
     ap.dbg = a.dbg;
     void* args[] = {(void*)&a, (void*)&ap};
-    const size_t smem = a.Xf ? (size_t)a.K * kFullSmem : 0;
+    const size_t smem = solve_smem(a, grid);
     // a continuation of a stopped solve runs its own instantiation
     const void* kern = a.resume ? (const void*)cocg_persistent<R, ApplyHubbard<W>, true>
                                 : (const void*)cocg_persistent<R, ApplyHubbard<W>, false>;
     if (smem > 0)   // above the 48 KB default together with the static part
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemMax);
     return cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(kBlock), args, smem, st);
 }
 template cudaError_t hubbard_launch_solve<double>(const SolveArgs<double>&, const Hubbard&, int, cudaStream_t);

@@ -469,12 +469,12 @@ cudaError_t hubbard2_launch_solve(const SolveArgs<R>& a, const Hubbard& hb, int 
     ApplyHubbard2<W> ap = make_apply2<W>(hb);
     ap.dbg = a.dbg;
     void* args[] = {(void*)&a, (void*)&ap};
-    const size_t smem = a.Xf ? (size_t)a.K * kFullSmem : 0;
+    const size_t smem = solve_smem(a, grid);
     // a continuation of a stopped solve runs its own instantiation
     const void* kern = a.resume ? (const void*)cocg_persistent<R, ApplyHubbard2<W>, true>
                                 : (const void*)cocg_persistent<R, ApplyHubbard2<W>, false>;
     if (smem > 0)   // above the 48 KB default together with the static part
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemMax);
     return cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(kBlock), args, smem, st);
 }
 template cudaError_t hubbard2_launch_solve<double>(const SolveArgs<double>&, const Hubbard&, int, cudaStream_t);

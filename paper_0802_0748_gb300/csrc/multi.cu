@@ -17,9 +17,11 @@ namespace scocg {
 namespace {
 
 template <typename R, class Apply>
-int multi_occupancy() {
+int multi_occupancy(size_t smem = 0) {
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, cocg_multi<R, Apply>, kBlock, 0) != cudaSuccess) return 0;
+    if (smem > 0)
+        cudaFuncSetAttribute((const void*)cocg_multi<R, Apply>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemMax);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, cocg_multi<R, Apply>, kBlock, smem) != cudaSuccess) return 0;
     return nb;
 }
 
@@ -77,6 +79,7 @@ struct MultiPlan {
     void* d_aps = nullptr;     // [nsys] Apply
     int* d_off = nullptr;      // [nsys + 1]
     int total_grid = 0;
+    size_t smem = 0;           // dynamic shared memory per CTA (every system's part of q, or 0)
     cudaGraphExec_t exec = nullptr;
     cudaGraph_t graph = nullptr;
     cudaStream_t cap = nullptr;   // capture stream (the handles' stream may be the legacy default stream)
@@ -158,6 +161,13 @@ int run_multi(int nsys, const scocg_handle* hs, const scocg_c128* const* shifts,
         std::vector<int> off(nsys + 1, 0);
         for (int s = 0; s < nsys; ++s) off[s + 1] = off[s] + g[s];
         P->total_grid = off[nsys];
+        // q in shared memory when every system's CTAs can hold their part
+        P->smem = 0;
+        for (int s = 0; s < nsys; ++s)
+            P->smem = std::max(P->smem, q_smem_bytes<R>(units[s], rows_per_unit(hs[s]->layout(false).kind), g[s]));
+        const int per_sm = (P->total_grid + h0->num_sms - 1) / h0->num_sms;
+        if (P->smem * per_sm > kQSmemPerSm || multi_occupancy<R, Apply>(P->smem) * h0->num_sms < P->total_grid)
+            P->smem = 0;
         std::vector<SolveArgs<R>> args(nsys);
         std::vector<Apply> aps(nsys);
         for (int s = 0; s < nsys && e == cudaSuccess; ++s) {
@@ -226,9 +236,11 @@ int run_multi(int nsys, const scocg_handle* hs, const scocg_c128* const* shifts,
             a.sync.status = &h->d_ctrl->status;
             a.sync.timeout_ns = (uint64_t)(h->opts.timeout_ms * 1e6);
             a.sync.nctas = grid;
+            a.pk = ctrl_packets(h->d_ctrl, grid, pvec != nullptr, M);
             a.stats = &h->d_ctrl->stats;
             a.G = reinterpret_cast<double2*>(G_out[s]);
             a.dbg = h->d_ctrl->dbg;
+            a.q_smem = P->smem > 0;
             args[s] = a;
             aps[s] = mk(L);
             P->hs.push_back(h);
@@ -271,7 +283,7 @@ int run_multi(int nsys, const scocg_handle* hs, const scocg_c128* const* shifts,
     // the launch: control blocks reset, then the cooperative kernel
     auto enqueue = [&](cudaStream_t qs) -> cudaError_t {
         cudaError_t e2 = cudaSuccess;
-        for (int s = 0; s < nsys && e2 == cudaSuccess; ++s) e2 = cudaMemsetAsync(hs[s]->d_ctrl, 0, sizeof(Ctrl), qs);
+        for (int s = 0; s < nsys && e2 == cudaSuccess; ++s) e2 = cudaMemsetAsync(hs[s]->d_ctrl, 0, kCtrlBytes, qs);
         if (e2 != cudaSuccess) return e2;
         const SolveArgs<R>* da = (const SolveArgs<R>*)P->d_args;
         const Apply* dp = (const Apply*)P->d_aps;
@@ -280,7 +292,7 @@ int run_multi(int nsys, const scocg_handle* hs, const scocg_c128* const* shifts,
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(P->total_grid);
         cfg.blockDim = dim3(kBlock);
-        cfg.dynamicSmemBytes = 0;
+        cfg.dynamicSmemBytes = P->smem;
         cfg.stream = qs;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeCooperative;

@@ -102,15 +102,20 @@ cudaError_t launch_csr(const SolveArgs<double>& a, const int* rowptr, const int*
                        int64_t n, int64_t nnz, int grid, cudaStream_t st) {
     ApplyCSRFixed<LPR> ap{{rowptr, col, val, n, nnz, a.dbg}};
     void* args[] = {(void*)&a, (void*)&ap};
-    return cudaLaunchCooperativeKernel((const void*)cocg_persistent<double, ApplyCSRFixed<LPR>>, dim3(grid),
-                                       dim3(kBlock), args, 0, st);
+    const void* kern = (const void*)cocg_persistent<double, ApplyCSRFixed<LPR>>;
+    const size_t smem = solve_smem(a, grid);
+    if (smem > 0) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemMax);
+    return cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(kBlock), args, smem, st);
 }
 
 template <int LPR>
-int occupancy_csr() {
+int occupancy_csr(size_t smem) {
     int nb = 0;
+    if (smem > 0)
+        cudaFuncSetAttribute((const void*)cocg_persistent<double, ApplyCSRFixed<LPR>>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemMax);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, cocg_persistent<double, ApplyCSRFixed<LPR>>, kBlock,
-                                                      0) != cudaSuccess)
+                                                      smem) != cudaSuccess)
         return 0;
     return nb;
 }
@@ -141,7 +146,10 @@ extern "C" int scocg_solve_csr_noalloc(int64_t n, int64_t nnz, const int32_t* ro
 
     const double avg = (double)nnz / (double)n;
     const int lpr = avg <= 4.0 ? 1 : (avg <= 24.0 ? 4 : 16);
-    const int occ = lpr == 1 ? occupancy_csr<1>() : (lpr == 4 ? occupancy_csr<4>() : occupancy_csr<16>());
+    auto occupancy = [&](size_t smem) {
+        return lpr == 1 ? occupancy_csr<1>(smem) : (lpr == 4 ? occupancy_csr<4>(smem) : occupancy_csr<16>(smem));
+    };
+    const int occ = occupancy(0);
     if (occ <= 0) return SCOCG_ERR_CUDA;
     const int rpu = 32 / lpr;
     const int64_t nunits = (n + rpu - 1) / rpu;
@@ -156,7 +164,7 @@ extern "C" int scocg_solve_csr_noalloc(int64_t n, int64_t nnz, const int32_t* ro
     SolveArgs<double> a{};
     Ctrl* ctrl = nullptr;
     auto carve = [&](Carver& c) {
-        ctrl = (Ctrl*)c.take(sizeof(Ctrl));
+        ctrl = (Ctrl*)c.take(grid > kPktCtas ? sizeof(Ctrl) : kCtrlBytes);
         a.r = (double2*)c.take(sizeof(double2) * (size_t)n);
         a.q = (double2*)c.take(sizeof(double2) * (size_t)n);
         a.cidx = proj_idx ? (const int64_t*)c.take(sizeof(int64_t) * M) : nullptr;
@@ -185,7 +193,8 @@ extern "C" int scocg_solve_csr_noalloc(int64_t n, int64_t nnz, const int32_t* ro
 
     // the control block (barrier counter, status, statistics) must start at
     // zero; everything else is written by the kernel before it is read
-    e = cudaMemsetAsync(ctrl, 0, sizeof(Ctrl), st);
+    a.pk = ctrl_packets(ctrl, grid, proj_vec != nullptr, M);
+    e = cudaMemsetAsync(ctrl, 0, a.pk ? kCtrlBytes : sizeof(Ctrl), st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync((void*)a.z, shifts, sizeof(double2) * K, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && proj_idx)
@@ -213,6 +222,9 @@ extern "C" int scocg_solve_csr_noalloc(int64_t n, int64_t nnz, const int32_t* ro
     a.stats = &ctrl->stats;
     a.G = reinterpret_cast<double2*>(G_out);
     a.dbg = ctrl->dbg;
+    const size_t qb = q_smem_bytes<double>(nunits, rpu, grid);
+    const int per_sm = (grid + sms - 1) / sms;
+    a.q_smem = qb * per_sm <= kQSmemPerSm && (int64_t)occupancy(qb) * sms >= grid;
 
     e = lpr == 1 ? launch_csr<1>(a, rowptr, col, val, n, nnz, grid, st)
       : lpr == 4 ? launch_csr<4>(a, rowptr, col, val, n, nnz, grid, st)

@@ -31,6 +31,7 @@ constexpr int kMaxProjB = 4;   // unit projections per right-hand side of a bloc
 #ifndef SCOCG_BSR4_GROUP
 #define SCOCG_BSR4_GROUP 4     // slots of the blocked apply whose loads are issued together
 #endif
+constexpr int kPktCtas = 64, kPktVals = 7;
 constexpr int kPartC = 10;   // active, best |pi|, arg, bad, pi_prev, pi_cur, alpha_k of arg
 
 struct ShiftState {          // device arrays, [K] or [K][M]
@@ -327,6 +328,11 @@ template <typename R> struct BsrApply { using T = ApplyBSR4<typename ValT<R>::T>
 template <> struct BsrApply<float> { using T = ApplyBSR4C<float>; };
 
 // ---------------------------------------------------------------- arguments
+// Dynamic shared memory of the full-vector mode with K shifts: per shift two
+// coefficients, the scale of its direction and a list entry, rounded so that
+// what follows is 16-byte aligned.
+__host__ __device__ inline size_t full_smem(int K) { return ((size_t)K * (3 * 16 + 4) + 15) / 16 * 16; }
+
 template <typename R>
 struct SolveArgs {
     using V = typename Vec<R>::T;
@@ -359,6 +365,9 @@ struct SolveArgs {
     double* partC;             // [grid][kPartC]
     int strideB;
     GridSync sync;
+    // packets of the partial sums, [kPktVals][grid] (phase A 2, phase B 5), or
+    // null: grid barriers (more than kPktCtas CTAs or dense projections)
+    ulonglong2* pk;
     SolveStats* stats;
     double2* G;                // out [nproj][K] for this right-hand side
     int debug_inject;
@@ -366,25 +375,44 @@ struct SolveArgs {
     int* trace;                // checked builds: host-mapped (iteration, phase) per CTA
     unsigned long long* phase_ns;  // phase-timer builds: [grid][8] accumulated ns
     // full-vector mode (FP64 only): per-shift solutions and directions, [K][n];
-    // needs K * kFullSmem bytes of dynamic shared memory
+    // needs full_smem(K) bytes of dynamic shared memory
     double2* Xf;
     double2* Pf;
     // continuation: the state a solve stopped at max_iter leaves (written at
     // exit when non-null), and resume = 1 to start from it instead of r_0 = b
     ResumeState* rstate;
     int resume;
+    // 1: q lives in dynamic shared memory (after the full-vector mode's part),
+    // [rows of the CTA]; a.q then only carries it to and from a continuation
+    int q_smem;
 };
-constexpr int kFullSmem = 3 * 16 + 4;   // per shift: two coefficients, the scale of its direction, a list entry
+
+// Dynamic shared memory of a solve's CTAs: the full-vector mode's shift
+// scalars, then the CTA's rows of q (at most ceil(nunits / grid) units).
+template <typename R>
+inline size_t q_smem_bytes(int64_t nunits, int rows_per_unit, int grid) {
+    return sizeof(typename Vec<R>::T) * (size_t)((nunits + grid - 1) / grid) * rows_per_unit;
+}
+template <typename R>
+inline size_t solve_smem(const SolveArgs<R>& a, int grid) {
+    return full_smem(a.Xf ? a.K : 0) + (a.q_smem ? q_smem_bytes<R>(a.nunits, a.rows_per_unit, grid) : 0);
+}
+// q is kept in shared memory while the CTAs of an SM hold at most this much of
+// it: the rest of the SM's 256 KB is the L1 that the gathers of the apply use.
+#ifndef SCOCG_Q_SMEM_PER_SM
+#define SCOCG_Q_SMEM_PER_SM (112 << 10)
+#endif
+constexpr size_t kQSmemPerSm = SCOCG_Q_SMEM_PER_SM;
+// Opt-in limit given to every solve kernel that uses dynamic shared memory: one
+// constant (the largest use: a CTA's q and 512 shifts of the full-vector mode),
+// so that solves in different threads cannot lower it under each other.
+constexpr int kDynSmemMax = (int)kQSmemPerSm + (32 << 10);
 
 // Shared per-CTA copy of the seed scalars; every CTA holds identical values.
-// CTA scratch of the block sums: per warp 3 + 2 kMaxProj values, or (FP64
-// block sums) kScratchNV values per thread
-constexpr int kScratchNV = 5;
-constexpr int kScratch = kWarps * (3 + 2 * kMaxProj) > kScratchNV * kBlock ? kWarps * (3 + 2 * kMaxProj)
-                                                                          : kScratchNV * kBlock;
+constexpr int kScratchNV = 5;   // values of one block sum
 struct SeedScalars {
     double2 alpha, alpha_prev, beta_prev, rho, rho_prev, zs;
-    double2 t2;                 // alpha_n beta_{n-1} / alpha_{n-1}
+    double2 inv_rho, t2_ratio;  // 1 / rho_n, beta_{n-1} / alpha_{n-1}
     double bnorm, inv_b2;       // ||b||, 1 / ||b||^2
     double2 beta_next;          // rho_{n+1} / rho_n, before it becomes beta_prev
     int seed, active, n;
@@ -393,7 +421,6 @@ struct SeedScalars {
     double2 cr_cur[kMaxProj];   // c_m^T r_n
     double2 cr_next[kMaxProj];  // c_m^T r_{n+1}
     double red[4 + 2 * kMaxProj + 4];
-    double scratch[kScratch];
 };
 
 }  // namespace scocg

@@ -11,19 +11,18 @@
 namespace scocg {
 
 // Dynamic shared memory above the 48 KB default (with the static part) needs
-// the kernel's opt-in; the full-vector mode asks for up to kMaxFullShifts x
-// kFullSmem bytes.
+// the kernel's opt-in (see solve_smem).
 template <typename R, class Apply, bool kResume = false>
 static void allow_dyn_smem(size_t smem) {
     if (smem > 0)
         cudaFuncSetAttribute((const void*)cocg_persistent<R, Apply, kResume>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemMax);
 }
 
 template <typename R, class Apply, bool kResume>
 static cudaError_t coop_launch(const SolveArgs<R>& a, const Apply& ap, int grid, cudaStream_t st) {
     void* args[] = {(void*)&a, (void*)&ap};
-    const size_t smem = a.Xf ? (size_t)a.K * kFullSmem : 0;
+    const size_t smem = solve_smem(a, grid);
     allow_dyn_smem<R, Apply, kResume>(smem);
     return cudaLaunchCooperativeKernel((const void*)cocg_persistent<R, Apply, kResume>, dim3(grid), dim3(kBlock),
                                        args, smem, st);

@@ -22,25 +22,40 @@ template <> __device__ __forceinline__ double unpark<dfs>(const double* slot) {
     return to_double(*reinterpret_cast<const dfs*>(slot));
 }
 
+// Where a CTA's partial sums of one reduction go: value j to part[j * G] (read
+// after a grid barrier), or, with pk set, to packet pk[j * G] = {value, tag}
+// that the other CTAs wait for directly (grids up to kPktCtas).
+struct PartialOut {
+    double* part;
+    ulonglong2* pk;
+    int G;
+    unsigned long long tag;
+    bool skip;               // fault injection: do not publish
+    __device__ __forceinline__ void put(int j, double t) const {
+        if (!pk) part[(size_t)j * G] = t;
+        else if (!skip) st_packet(pk + (size_t)j * G, t, tag);
+    }
+};
+
 // CTA sums of the first nv of NV per-thread values, of which only the warps
-// with place wi < nw hold any: warp j < nv writes sum j to part[j * G] (the caller
-// synchronises the CTA before anyone reads it or reuses scratch).  Each sum is
-// a tree, not a chain: a serial FP64 chain over 16 warps was ~0.5 us of every
-// seed iteration, twice.
-template <int NV, typename T>
-__device__ __forceinline__ void block_partials(T (&v)[NV], double* scratch, double* part, int G, int wi,
+// with place wi < nw hold any: warp j < nv publishes sum j (the caller
+// synchronises the CTA before anyone reuses scratch).  Each sum is a tree, not
+// a chain: a serial FP64 chain over 16 warps was ~0.5 us of every seed
+// iteration, twice.
+template <int NV, typename T, int kScratch>
+__device__ __forceinline__ void block_partials(T (&v)[NV], double (&scratch)[kScratch], const PartialOut& out, int wi,
                                                int nv = NV, int nw = kWarps) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    static_assert(kScratch >= NV * (std::is_same<T, double>::value ? kBlock : kWarps), "scratch too small");
     if constexpr (std::is_same<T, double>::value) {
-        // FP64 values: every thread parks its values (scratch holds NV *
-        // kBlock doubles) and nv warps sum them, instead of five-step FP64
-        // warp sums in all warps
-        static_assert(NV <= kScratchNV, "scratch too small");
+        // FP64 values: every thread parks its values and nv warps sum them,
+        // instead of five-step FP64 warp sums in all warps
         if (wi < nw)
 #pragma unroll
             for (int j = 0; j < NV; ++j)
                 if (j < nv) scratch[j * kBlock + 32 * wi + lane] = v[j];
         __syncthreads();
+        if (out.pk && warp < nv && lane == 0) fence_acq_rel();   // the CTA's writes come before its packets
         if (warp < nv) {
             double a[4] = {0.0, 0.0, 0.0, 0.0};
             for (int w = 0; w < nw; w += 4)
@@ -53,7 +68,7 @@ __device__ __forceinline__ void block_partials(T (&v)[NV], double* scratch, doub
             if (nw > 2) { a[0] += a[2]; if (nw > 3) a[1] += a[3]; }
             if (nw > 1) a[0] += a[1];
             const double t = warp_sum(a[0]);
-            if (lane == 0) part[(size_t)warp * G] = t;
+            if (lane == 0) out.put(warp, t);
         }
     } else {
         // the warp-level part in the values' own type, the sum over warps in FP64
@@ -64,11 +79,12 @@ __device__ __forceinline__ void block_partials(T (&v)[NV], double* scratch, doub
             if (lane == 0) park(scratch + j * kWarps + wi, t);
         }
         __syncthreads();
+        if (out.pk && warp < nv && lane == 0) fence_acq_rel();
         if (warp < nv) {
             double t = lane < kWarps ? unpark<T>(scratch + warp * kWarps + lane) : 0.0;
 #pragma unroll
             for (int o = kWarps / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-            if (lane == 0) part[(size_t)warp * G] = t;
+            if (lane == 0) out.put(warp, t);
         }
     }
 }
@@ -156,33 +172,80 @@ __device__ __forceinline__ float4 r_update<float4>(float4 r, float4 al, float4 q
     return vcfma(make_float4(-al.x, -al.y, -al.z, -al.w), q, r);
 }
 
+// A CTA's share of the rows and where its part of q lives.  Its units are
+// numbered lu = 0 .. nloc - 1 and its rows t = 0 .. nrow - 1; every phase of an
+// iteration gives a row to the same CTA, so q, which only the row's owner
+// reads, can stay in shared memory (on): it is then neither written to nor read
+// from L2, and the first reduction's release has no vector stores to wait for.
+// A strided apply (Hubbard, q in global memory) uses contiguous rows in the
+// row-wise phases.
+template <class Apply, typename V>
+struct RowShare {
+    static constexpr bool kStrided = Apply::kMap == kMapStrided;
+    static constexpr int kRpu = Apply::kRowsPerUnit;
+    int G, cta, nloc, nrow;
+    int64_t ubeg, rbeg;
+    bool on;
+    V* q_s;
+    V* q_g;
+    __device__ __forceinline__ RowShare(int64_t n, int64_t nunits, int G_, int cta_, bool on_, V* qs, V* qg)
+        : G(G_), cta(cta_), on(!kStrided && on_), q_s(qs), q_g(qg) {
+        if constexpr (kStrided) {
+            ubeg = cta;
+            nloc = cta < nunits ? (int)((nunits - cta + G - 1) / G) : 0;
+            rbeg = (int64_t)cta * n / G;
+            nrow = (int)((int64_t)(cta + 1) * n / G - rbeg);
+        } else {
+            ubeg = (int64_t)cta * nunits / G;
+            nloc = (int)((int64_t)(cta + 1) * nunits / G - ubeg);
+            rbeg = ubeg * kRpu;
+            nrow = (int)(min(n, rbeg + (int64_t)nloc * kRpu) - rbeg);
+        }
+    }
+    __device__ __forceinline__ int64_t unit(int lu) const { return kStrided ? ubeg + (int64_t)G * lu : ubeg + lu; }
+    __device__ __forceinline__ int64_t row(int t) const { return rbeg + t; }
+    // place of the row that `lane` owns in unit lu
+    __device__ __forceinline__ int place(int lu, int lane) const { return lu * kRpu + lane / (32 / kRpu); }
+    __device__ __forceinline__ V get(int t, int64_t r) const { return on ? q_s[t] : q_g[r]; }
+    __device__ __forceinline__ void put(int t, int64_t r, V v) const {
+        if (on) q_s[t] = v; else q_g[r] = v;
+    }
+};
+
 // CTA sums of the accumulated partials into values 0..2 (0..4 with dense
 // projections) of this CTA's column of the value-major partials (value j at
 // part[j * G]); the extra dense projections m >= 1 are summed in separate
 // passes over r into values 3 + 2m.
-template <typename R>
+template <typename R, class Share, int kScratch>
 __device__ __forceinline__ void finish_r_partials(const SolveArgs<R>& a, typename Acc<R>::T (&acc)[5],
-                                                  int64_t rbeg, int64_t rend, SeedScalars& s, double* part, int G) {
+                                                  const Share& sh, double (&scratch)[kScratch],
+                                                  const PartialOut& out) {
     using AT = typename Acc<R>::T;
     const int tid = threadIdx.x;
-    const int nw = (int)min((int64_t)kWarps, (rend - rbeg + 31) >> 5);   // warps that hold rows
+    const int nw = min(kWarps, (sh.nrow + 31) >> 5);   // warps that hold rows
     end_rr(acc[0], acc[1], acc[2]);
-    block_partials<5>(acc, s.scratch, part, G, tid >> 5, a.cvec ? 5 : 3, max(nw, 1));
+    block_partials<5>(acc, scratch, out, tid >> 5, a.cvec ? 5 : 3, max(nw, 1));
     for (int m = 1; m < a.nproj && a.cvec; ++m) {
         AT w2[2] = {};
-        for (int64_t i = rbeg + tid; i < rend; i += kBlock) acc_bil(w2[0], w2[1], a.cvec[(size_t)m * a.n + i], a.r[i]);
+        for (int t = tid; t < sh.nrow; t += kBlock) {
+            const int64_t i = sh.row(t);
+            acc_bil(w2[0], w2[1], a.cvec[(size_t)m * a.n + i], a.r[i]);
+        }
         __syncthreads();   // the sums above have been read from scratch
-        block_partials<2>(w2, s.scratch, part + (size_t)(3 + 2 * m) * G, G, tid >> 5, 2, max(nw, 1));
+        const PartialOut om{out.part + (size_t)(3 + 2 * m) * out.G, nullptr, out.G, 0ull, false};   // more than one: no packets
+        block_partials<2>(w2, scratch, om, tid >> 5, 2, max(nw, 1));
     }
 }
 
-template <typename R>
-__device__ __forceinline__ void r_partials(const SolveArgs<R>& a, int64_t rbeg, int64_t rend,
-                                           SeedScalars& s, double* part, int G) {
+template <typename R, class Share, int kScratch>
+__device__ __forceinline__ void r_partials(const SolveArgs<R>& a, const Share& sh, double (&scratch)[kScratch],
+                                           const PartialOut& out) {
     typename Acc<R>::T acc[5] = {};
-    for (int64_t i = rbeg + threadIdx.x; i < rend; i += kBlock)
+    for (int t = threadIdx.x; t < sh.nrow; t += kBlock) {
+        const int64_t i = sh.row(t);
         acc_r<R>(acc, a.r[i], a.cvec ? a.cvec + i : nullptr);
-    finish_r_partials(a, acc, rbeg, rend, s, part, G);
+    }
+    finish_r_partials(a, acc, sh, scratch, out);
 }
 
 #ifdef SCOCG_CHECKED
@@ -225,36 +288,52 @@ struct ShiftInputs {
     double2 cr[kMaxProj];
 };
 
-// Phase C for shift k: the pi three-term recurrence, the projected p^k and
-// x^k, the residual estimate and freezing.  Sets bad for a zero or non-finite
-// pi, active when the shift stays unconverged.
-template <typename R>
-__device__ __forceinline__ void shift_update(const SolveArgs<R>& a, int k, const ShiftInputs& c, int M,
+// The per-shift state of a CTA's own shifts in shared memory, one slot per
+// owning thread: each seed iteration reads and writes it once, and a global
+// load after a grid barrier is a round trip to L2 (300 to 800 cycles).  Used
+// when every owner is in warp 0 and a shift has at most kOwnM projections; the
+// state is copied to the global arrays at the end of the solve.
+constexpr int kOwn = 32, kOwnM = 2;
+struct OwnShifts {
+    double2 pi_prev[kOwn], pi_cur[kOwn], sigma[kOwn], alpha_k[kOwn], inv_cur[kOwn];
+    double2 P[kOwn * kOwnM], X[kOwn * kOwnM];
+    double resid[kOwn];
+    int frozen[kOwn], iters[kOwn];
+};
+__device__ __forceinline__ ShiftState own_view(OwnShifts& o) {
+    return ShiftState{o.pi_prev, o.pi_cur, o.sigma, o.alpha_k, o.inv_cur, o.P, o.X, o.frozen, o.iters, o.resid};
+}
+
+// Phase C for the shift in slot k of S: the pi three-term recurrence, the
+// projected p^k and x^k, the residual estimate and freezing.  Sets bad for a
+// zero or non-finite pi (its state is then left as it was), active when the
+// shift stays unconverged.
+__device__ __forceinline__ void shift_update(const ShiftState& S, int k, const ShiftInputs& c, int M, double tol,
                                              double tol2, int& active, int& bad) {
-    const double2 pp = a.S.pi_prev[k], pc = a.S.pi_cur[k], ic = a.S.inv_cur[k];
+    const double2 pp = S.pi_prev[k], pc = S.pi_cur[k], ic = S.inv_cur[k];
+    const double2 pn = cadd(cmul(cadd(c2(1, 0), cmul(c.alpha, S.sigma[k])), pc), cmul(c.t2, csub(pc, pp)));
+    const double2 in = crecip(pn);
     const double2 ratio = cmul(pp, ic);                        // pi_{n-1} / pi_n
     const double2 beta_k = cmul(cmul(ratio, ratio), c.beta_prev);
-    const double2 pn = cadd(cmul(cadd(c2(1, 0), cmul(c.alpha, a.S.sigma[k])), pc), cmul(c.t2, csub(pc, pp)));
-    const double2 in = crecip(pn);
+    const double2 ak = cmul(cmul(pc, in), c.alpha);            // alpha^k_n
+    const double res2 = c.rn_b2 * cabs2(in);
     if (cabs2(pn) == 0.0 || !cfinite(pn) || !cfinite(in)) {
         bad = 1;
         return;
     }
-    const double2 ak = cmul(cmul(pc, in), c.alpha);            // alpha^k_n
     for (int m = 0; m < M; ++m) {
         const size_t o = (size_t)k * M + m;
-        const double2 P = cadd(cmul(c.cr[m], ic), cmul(beta_k, a.S.P[o]));
-        a.S.P[o] = P;
-        a.S.X[o] = cadd(a.S.X[o], cmul(ak, P));
+        const double2 P = cadd(cmul(c.cr[m], ic), cmul(beta_k, S.P[o]));
+        S.P[o] = P;
+        S.X[o] = cadd(S.X[o], cmul(ak, P));
     }
-    a.S.alpha_k[k] = ak;
-    a.S.pi_prev[k] = pc;
-    a.S.pi_cur[k] = pn;
-    a.S.inv_cur[k] = in;
-    const double res2 = c.rn_b2 * cabs2(in);
-    a.S.resid[k] = res2;
-    a.S.iters[k] = c.n + 1;
-    if (a.tol > 0.0 && res2 <= tol2) a.S.frozen[k] = 1;
+    S.alpha_k[k] = ak;
+    S.pi_prev[k] = pc;
+    S.pi_cur[k] = pn;
+    S.inv_cur[k] = in;
+    S.resid[k] = res2;
+    S.iters[k] = c.n + 1;
+    if (tol > 0.0 && res2 <= tol2) S.frozen[k] = 1;
     else active = 1;
 }
 
@@ -285,26 +364,195 @@ __device__ __forceinline__ void sum_counts(const double* part, int G, int& activ
     bad = __reduce_or_sync(0xffffffffu, any);
 }
 
+// A packet's tag: the reduction's number in the low word; phase A's first
+// packet carries the CTA's shift counts in the high word.
+__device__ __forceinline__ unsigned long long packet_tag(unsigned no, int active, int bad) {
+    return ((unsigned long long)((unsigned)active | (bad ? 0x80000000u : 0u)) << 32) | no;
+}
+
+// Waits for nv packets of each of the G CTAs (warp j < nv for packet j, two
+// CTAs per lane) and leaves their sums, the same in every CTA, in out[0..nv)
+// and the counts of packet 0 in counts[0..1] (counts[2]: a wait was given up).  One round trip through L2
+// instead of the barrier's arrival, its poll and then the loads of the
+// partials (32 CTAs: 1.1 us against 1.25 + 0.6).  A packet is rewritten only
+// after a later reduction that every CTA takes part in.  The wait is bounded
+// like the grid barrier's; false ends the solve.
+__device__ __forceinline__ bool packet_sums(const GridSync& g, const ulonglong2* pk, int G, int nv, unsigned no,
+                                            double* out, int* counts) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp < nv) {
+        double v[2] = {0.0, 0.0};
+        unsigned aux = 0u, any = 0u;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int c = lane + 32 * h;
+            if (c >= G) break;
+            unsigned long long tag = 0;
+            uint64_t t0 = 0;
+            for (unsigned turn = 1;; ++turn) {
+                v[h] = ld_packet(pk + (size_t)warp * G + c, tag);
+                if ((unsigned)tag == no) break;
+                if (turn & 63u) continue;
+                const uint64_t t = globaltimer_ns();
+                if (t0 == 0) t0 = t;
+                if (ld_volatile_i32(g.status) < 0 || t - t0 > g.timeout_ns) {
+                    atomicCAS(g.status, 0, (int)SCOCG_ERR_TIMEOUT);
+                    atomicCAS(g.status, 1, (int)SCOCG_ERR_TIMEOUT);
+                    counts[2] = 1;
+                    break;
+                }
+            }
+            aux += (unsigned)(tag >> 32) & 0x7fffffffu;
+            any |= (unsigned)(tag >> 63);
+        }
+        __syncwarp();
+        fence_acq_rel();   // the CTA's later loads see the writes before the packets
+        const double t = warp_sum(G > 32 ? v[0] + v[1] : v[0]);
+        if (lane == 0) out[warp] = t;
+        if (warp == 0) {
+            aux = __reduce_add_sync(0xffffffffu, aux);
+            any = __reduce_or_sync(0xffffffffu, any);
+            if (lane == 0) { counts[0] = (int)aux; counts[1] = (int)any; }
+        }
+    }
+    __syncthreads();
+    return counts[2] == 0;
+}
+
+// Order in which the warps take units when warps 0 and 1 first do scalar work:
+// they get the last two places of each round.
+__device__ __forceinline__ int rotated_place(int warp) { return (warp + kWarps - 2) % kWarps; }
+
+// a / b by one warp (all lanes return it): the products a conj(b) and |b|^2
+// run in different lanes of the same instructions.  A warp issues an FP64
+// instruction every 64 cycles however few lanes are active, so the serial time
+// of scalar code is its instruction count (cdiv: 17 of them, here 10).
+__device__ __forceinline__ double2 warp_cdiv(double2 a, double2 b) {
+    const int role = threadIdx.x & 3;
+    const int e = max(__double2hiint(b.x) & 0x7ff00000, __double2hiint(b.y) & 0x7ff00000) >> 20;
+    if (e < 1023 - 400 || e > 1023 + 400) return cdiv(a, b);   // |b|^2 needs scaling (uniform)
+    const double u = role == 0 ? a.x : role == 1 ? a.y : b.x;
+    const double v = role == 0 ? a.y : role == 1 ? -a.x : b.y;
+    const double p = fma(u, b.x, v * b.y);     // a.x b.x + a.y b.y | a.y b.x - a.x b.y | |b|^2
+    const double inv = __drcp_rn(__shfl_sync(0xffffffffu, p, 2));
+    const double y = p * inv;
+    return c2(__shfl_sync(0xffffffffu, y, 0), __shfl_sync(0xffffffffu, y, 1));
+}
+// one component (cc = 0: real, 1: imaginary) of a b + c
+__device__ __forceinline__ double cfma_part(double2 a, double2 b, int cc, double c) {
+    return fma(a.x, cc ? b.y : b.x, fma(a.y, cc ? b.x : -b.y, c));
+}
+// the lane pair's complex number from each lane's component
+__device__ __forceinline__ double2 pair_of(double part, int cc) {
+    const double o = __shfl_xor_sync(0xffffffffu, part, 1);
+    return cc ? c2(o, part) : c2(part, o);
+}
+// rho_new / rho from inv = 1 / rho (known before rho_new), with one correction
+// step: two lanes of a warp, six FP64 instructions.
+__device__ __forceinline__ double2 warp_quot(double2 a, double2 b, double2 inv) {
+    const int cc = threadIdx.x & 1;
+    const double2 y = pair_of(cfma_part(a, inv, cc, 0.0), cc);
+    const double2 r = pair_of(cfma_part(c2(-y.x, -y.y), b, cc, cc ? a.y : a.x), cc);
+    return pair_of(cfma_part(r, inv, cc, cc ? y.y : y.x), cc);
+}
+
+// Phase C for the CTA's nown shifts in shared memory, by one warp: eight lanes
+// per shift, four shifts at a time, the independent products of the update in
+// lane pairs of the same instructions (24 FP64 instructions instead of ~80 in
+// one lane; see warp_cdiv).  Lane pair g = 0: pi and its reciprocal, 1:
+// beta^k, 2 and 3: the projections; lane cc of a pair: real or imaginary part.
+__device__ __forceinline__ void shift_update_warp(OwnShifts& o, int nown, const ShiftInputs& c, int M, double tol,
+                                                  double tol2, int& active, int& bad) {
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31, g = (lane >> 1) & 3, cc = lane & 1, b8 = lane & 24;
+    int act = 0, bd = 0;
+    for (int k0 = 0; k0 < nown; k0 += 4) {
+        const int kk = k0 + (lane >> 3);
+        const bool live = kk < nown && !o.frozen[kk];
+        if (!__any_sync(kAll, live)) continue;
+        const int k = kk < nown ? kk : 0;
+        const double2 pp = o.pi_prev[k], pc = o.pi_cur[k], ic = o.inv_cur[k];
+        const int m = g == 2 ? 1 : 0;                      // the projection of pair g = 3 (0) or 2 (1)
+        const bool has_p = g == 3 || (g == 2 && M > 1);
+        const double2 Po = has_p ? o.P[k * M + m] : c2(0, 0), Xo = has_p ? o.X[k * M + m] : c2(0, 0);
+        const double2 cr1 = M > 1 ? c.cr[1] : c2(0, 0);
+        // 1 + alpha sigma | pi_{n-1} / pi_n | t2 (pi_n - pi_{n-1}) | c_0^T r / pi_n
+        const double2 A1 = g == 0 ? c.alpha : g == 1 ? pp : g == 2 ? c.t2 : c.cr[0];
+        const double2 B1 = g == 0 ? o.sigma[k] : g == 2 ? csub(pc, pp) : ic;
+        const double s1 = cfma_part(A1, B1, cc, g == 0 && cc == 0 ? 1.0 : 0.0);
+        const double2 U = pair_of(s1, cc);
+        const double v = __shfl_sync(kAll, s1, b8 | 4 | cc);
+        // pi_{n+1} | (pi_{n-1} / pi_n)^2 | c_1^T r / pi_n
+        const double2 A2 = g == 2 ? cr1 : U, B2 = g == 0 ? pc : g == 1 ? U : ic;
+        const double s2 = cfma_part(A2, B2, cc, g == 0 ? v : 0.0);
+        const double2 W = pair_of(s2, cc);
+        // |pi_{n+1}|^2 | beta^k
+        const double b1 = g == 0 ? W.x : cc ? c.beta_prev.y : c.beta_prev.x;
+        const double b2 = g == 0 ? W.y : cc ? c.beta_prev.x : -c.beta_prev.y;
+        const double s3 = fma(W.x, b1, W.y * b2);
+        const double d = __shfl_sync(kAll, s3, b8);
+        const double2 pn = c2(__shfl_sync(kAll, s2, b8), __shfl_sync(kAll, s2, b8 | 1));
+        const double2 bk = c2(__shfl_sync(kAll, s3, b8 | 2), __shfl_sync(kAll, s3, b8 | 3));
+        const double Pn = cfma_part(bk, Po, cc, g == 3 ? s1 : s2);        // p^k_m (pairs 2, 3)
+        const double2 Pc = pair_of(Pn, cc);
+        const int e = max(__double2hiint(pn.x) & 0x7ff00000, __double2hiint(pn.y) & 0x7ff00000) >> 20;
+        const bool plain = e >= 1023 - 400 && e <= 1023 + 400;            // |pi|^2 and its reciprocal in range
+        const double inv = __drcp_rn(d);
+        const double2 in = pair_of((cc ? -pn.y : pn.x) * inv, cc);
+        const double2 w = pair_of(cfma_part(pc, in, cc, 0.0), cc);
+        const double2 ak = pair_of(cfma_part(w, c.alpha, cc, 0.0), cc);   // alpha^k_n
+        const double Xn = cfma_part(ak, Pc, cc, cc ? Xo.y : Xo.x);
+        const double res2 = c.rn_b2 * inv;
+        __syncwarp();                                                     // every lane has read the old state
+        if (live && plain) {
+            double* P = reinterpret_cast<double*>(o.P + k * M + m);
+            double* X = reinterpret_cast<double*>(o.X + k * M + m);
+            if (has_p) { P[cc] = Pn; X[cc] = Xn; }
+            if (g == 0) reinterpret_cast<double*>(o.alpha_k + k)[cc] = cc ? ak.y : ak.x;
+            if (g == 1) reinterpret_cast<double*>(o.inv_cur + k)[cc] = cc ? in.y : in.x;
+            if (g == 0) {
+                reinterpret_cast<double*>(o.pi_prev + k)[cc] = cc ? pc.y : pc.x;
+                reinterpret_cast<double*>(o.pi_cur + k)[cc] = cc ? pn.y : pn.x;
+            }
+            if ((lane & 7) == 0) {
+                o.resid[k] = res2;
+                o.iters[k] = c.n + 1;
+                if (tol > 0.0 && res2 <= tol2) o.frozen[k] = 1;
+                else act = 1;
+            }
+        } else if (live && (lane & 7) == 0) {
+            int a1 = 0, b1_ = 0;
+            shift_update(own_view(o), k, c, M, tol, tol2, a1, b1_);
+            act = a1;
+            bd |= b1_;
+        }
+        active += __popc(__ballot_sync(kAll, act));
+        act = 0;
+        __syncwarp();
+    }
+    bad |= __any_sync(kAll, bd);
+}
+
 // The first phase A of a solve continued from a ResumeState: the stopped
 // apply's r^T q partial again, from the stored r_n and q_n over the same rows
 // in the same order (so the continued solve matches an uninterrupted one bit
 // for bit), and the shift count as its deferred phase C left it.
-template <typename R, class Apply>
-__device__ __forceinline__ void resume_partials(const SolveArgs<R>& a, const Apply& ap, int G, int cta, int64_t ubeg,
-                                             int64_t u_end, int64_t u_step, int nwA, bool active, SeedScalars& s) {
+template <typename R, class Apply, class Share, int kScratch>
+__device__ __forceinline__ void resume_partials(const SolveArgs<R>& a, const Apply& ap, const Share& sh, int nwA,
+                                             bool active, double (&scratch)[kScratch], const PartialOut& out) {
     using AT = typename Acc<R>::T;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const bool rot = a.rstate->rotated != 0;
-    const int wi = rot ? (warp + kWarps - 1) % kWarps : warp;
-    const int64_t first = Apply::kMap == kMapStrided ? (int64_t)cta + (int64_t)G * wi : ubeg + wi;
+    const int wi = a.rstate->rotated != 0 ? rotated_place(warp) : warp;
     AT rq[2] = {};
-    for (int64_t u = first; u < u_end; u += u_step) {
+    for (int lu = wi; lu < sh.nloc; lu += kWarps) {
         int64_t row;
-        if (ap.row_of(u, lane, row)) acc_bil(rq[0], rq[1], a.r[row], a.q[row]);
+        if (ap.row_of(sh.unit(lu), lane, row)) acc_bil(rq[0], rq[1], a.r[row], sh.get(sh.place(lu, lane), row));
     }
     const int act = __syncthreads_count(active);
-    block_partials<2>(rq, s.scratch, a.partA + cta, G, wi, 2, nwA);
-    if (tid == 64) a.partA[2 * G + cta] = pack_counts(act, 0);
+    PartialOut o = out;
+    o.tag = packet_tag((unsigned)out.tag, act, 0);
+    block_partials<2>(rq, scratch, o, wi, 2, nwA);
+    if (tid == 64) a.partA[2 * sh.G + sh.cta] = pack_counts(act, 0);
     __syncthreads();
 }
 
@@ -334,10 +582,15 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
     constexpr bool kMixed = std::is_same<R, float>::value;   // complex64 vectors
     constexpr bool kFull = std::is_same<R, double>::value;   // full-vector mode compiled (FP64 only)
     __shared__ SeedScalars s;
-    __shared__ int s_flag[7];            // 0, 1: this CTA's shift counts; 2, 3: decision; 4: seed converged; 5, 6: grid counts
+    __shared__ int s_flag[8];            // 0, 1: this CTA's shift counts; 2, 3: decision; 4: seed converged; 5, 6: grid counts; 7: lost
     __shared__ double s_min[kWarps];
     __shared__ int s_arg[kWarps];
     __shared__ ShiftInputs s_c;          // inputs of a deferred phase C
+    __shared__ OwnShifts s_own;
+    // block_partials: five sums over the rows, in FP64 over threads, else over
+    // warps (and one FP64 sum over threads, ||b||^2)
+    __shared__ double s_scratch[kFull ? kScratchNV * kBlock : kBlock];
+    __shared__ int64_t s_cidx[kMaxProj];
     // z_s, beta_{n-1}, alpha_n in the vector type, converted once by thread 0
     // whenever they change (every thread converting them would queue all
     // warps on the FP64 pipe at each phase start)
@@ -347,18 +600,12 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
 
     const int tid = threadIdx.x;
     const int lane = tid & 31, warp = tid >> 5;
-    // phase A visits units in the apply's order (kMap); the row-wise phases
-    // use a contiguous row range per CTA.
-    const int64_t ubeg = (int64_t)cta * a.nunits / G, uend = (int64_t)(cta + 1) * a.nunits / G;
-    constexpr bool kWhole = Apply::kMap != kMapContiguous;   // every CTA visits the whole unit range
-    const int64_t u_first = Apply::kMap == kMapStrided ? (int64_t)cta + (int64_t)G * warp : ubeg + warp;
-    const int64_t u_step = kWhole ? (int64_t)G * kWarps : kWarps;
-    const int64_t u_end = kWhole ? a.nunits : uend;
+    // phase A visits units in the apply's order (kMap)
+    const RowShare<Apply, V> sh(a.n, a.nunits, G, cta, a.q_smem != 0,
+                                reinterpret_cast<V*>(reinterpret_cast<char*>(s_full) + full_smem(a.Xf ? a.K : 0)),
+                                a.q);
     // warps that visit a unit (all of them when there are enough)
-    const int64_t u_cnt = Apply::kMap == kMapStrided ? (a.nunits - cta + G - 1) / G
-                          : kWhole ? a.nunits : uend - ubeg;
-    const int nwA = (int)max((int64_t)1, min((int64_t)kWarps, u_cnt));
-    const int64_t rbeg = (int64_t)cta * a.n / G, rend = (int64_t)(cta + 1) * a.n / G;
+    const int nwA = max(1, min(kWarps, sh.nloc));
     const int M = a.nproj;
     const bool dense_proj = a.cvec != nullptr;
     const int nred = dense_proj ? 3 + 2 * M : 3;
@@ -374,6 +621,23 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
     // seed has converged runs phase C in place.
     bool defer_ok = a.K <= 32 * G;
     if constexpr (kFull) defer_ok = defer_ok && a.Xf == nullptr;
+    // the own shifts' state: in shared memory where it fits (OwnShifts)
+    const bool own_sm = defer_ok && M <= kOwnM;
+    auto state = [&]() { return own_sm ? own_view(s_own) : a.S; };
+    const int ko = own_sm ? tid : k_own;      // this thread's slot in it
+    auto update_own = [&](int& act, int& bad) {
+        if (own_sm) shift_update(own_view(s_own), tid, s_c, M, a.tol, tol2, act, bad);
+        else shift_update(a.S, k_own, s_c, M, a.tol, tol2, act, bad);
+    };
+    const int nown = min(kOwn, (a.K - cta + G - 1) / G);   // the CTA's own shifts (own_sm: all of them)
+    // few own shifts: eight lanes each (three passes of ~24 FP64 instructions
+    // at most); more: one lane each (~80)
+    const bool own_wide = own_sm && nown <= 12;
+    if (tid < M && !dense_proj) s_cidx[tid] = a.cidx[tid];
+    // small grids exchange their partial sums as packets (packet_sums)
+    const bool pkt = a.pk != nullptr;
+    unsigned red_no = 0;                      // number of the last packet reduction
+    const PartialOut outB{myB, nullptr, G, 0ull, false};
     bool pending = false;                     // a deferred phase C waits for the next phase A
 
     int status = SCOCG_NOT_CONVERGED;
@@ -399,18 +663,35 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
             s.shift_iters = 0;
         }
         if (tid < M) s.cr_cur[tid] = a.rstate->cr_cur[tid];
+        const ShiftState S = state();
+        if (own_sm && owns) {
+            S.pi_prev[ko] = a.S.pi_prev[k_own]; S.pi_cur[ko] = a.S.pi_cur[k_own]; S.inv_cur[ko] = a.S.inv_cur[k_own];
+            S.sigma[ko] = a.S.sigma[k_own]; S.alpha_k[ko] = a.S.alpha_k[k_own];
+            for (int m = 0; m < M; ++m) {
+                S.P[ko * M + m] = a.S.P[(size_t)k_own * M + m];
+                S.X[ko * M + m] = a.S.X[(size_t)k_own * M + m];
+            }
+            S.frozen[ko] = a.S.frozen[k_own]; S.iters[ko] = a.S.iters[k_own]; S.resid[ko] = a.S.resid[k_own];
+        }
         // s_flag[4] (seed converged) decides whether the next apply takes a
         // deferred shift update and visits its units rotated: restored so
         // that a stop right after this pass records the stopped one's order
-        if (tid < 5) s_flag[tid] = tid == 4 ? (a.rstate->rotated ? 0 : 1) : 0;
+        if (tid < 8) s_flag[tid] = tid == 4 ? (a.rstate->rotated ? 0 : 1) : 0;
         __syncthreads();
-        resume_partials(a, ap, G, cta, ubeg, u_end, u_step, nwA, owns && !a.S.frozen[k_own], s);
+        if (sh.on) {
+            for (int t = tid; t < sh.nrow; t += kBlock) sh.q_s[t] = a.q[sh.row(t)];
+            __syncthreads();
+        }
+        resume_partials(a, ap, sh, nwA, owns && !S.frozen[ko], s_scratch,
+                         PartialOut{a.partA + cta, pkt ? a.pk + cta : nullptr, G, (unsigned long long)(++red_no), false});
     } else {
         double nb = 0.0;
-        for (int64_t i = rbeg + tid; i < rend; i += kBlock) {
+        const ShiftState S = state();
+        for (int t = tid; t < sh.nrow; t += kBlock) {
+            const int64_t i = sh.row(t);
             const double2 bi = a.b[i];
             a.r[i] = Vec<R>::make(bi);
-            a.q[i] = vzero<V>();
+            sh.put(t, i, vzero<V>());
             if constexpr (kMixed) {
                 a.p_seed[i] = vzero<V>(); a.x_hi[i] = vzero<V>(); a.x_lo[i] = vzero<V>();
             }
@@ -420,18 +701,17 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
             nb = fma(bi.x, bi.x, fma(bi.y, bi.y, nb));
         }
         double v1[1] = {nb};
-        block_partials<1>(v1, s.scratch, a.partC + (size_t)cta * kPartC, G, warp);
+        block_partials<1>(v1, s_scratch, PartialOut{a.partC + (size_t)cta * kPartC, nullptr, G, 0ull, false}, warp);
         __syncthreads();
-        r_partials(a, rbeg, rend, s, myB, G);
+        r_partials(a, sh, s_scratch, outB);
         if (owns) {
-            const int k = k_own;
-            a.S.pi_prev[k] = c2(1, 0); a.S.pi_cur[k] = c2(1, 0); a.S.inv_cur[k] = c2(1, 0);
-            a.S.sigma[k] = csub(a.z[k], a.z[a.seed]);
-            a.S.alpha_k[k] = c2(0, 0);
-            for (int m = 0; m < M; ++m) { a.S.P[(size_t)k * M + m] = c2(0, 0); a.S.X[(size_t)k * M + m] = c2(0, 0); }
-            a.S.frozen[k] = 0; a.S.iters[k] = 0; a.S.resid[k] = 1.0;
+            S.pi_prev[ko] = c2(1, 0); S.pi_cur[ko] = c2(1, 0); S.inv_cur[ko] = c2(1, 0);
+            S.sigma[ko] = csub(a.z[k_own], a.z[a.seed]);
+            S.alpha_k[ko] = c2(0, 0);
+            for (int m = 0; m < M; ++m) { S.P[(size_t)ko * M + m] = c2(0, 0); S.X[(size_t)ko * M + m] = c2(0, 0); }
+            S.frozen[ko] = 0; S.iters[ko] = 0; S.resid[ko] = 1.0;
         }
-        if (tid < 7) s_flag[tid] = 0;
+        if (tid < 8) s_flag[tid] = 0;
         if (!grid_barrier(a.sync, epoch)) return;
         grid_sum_vm1(a.partB, nred, s.red, G);
         grid_sum(a.partC, kPartC, 1, s.red + nred, G);
@@ -452,17 +732,25 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
         }
         if (tid < M) {
             s.cr_cur[tid] = dense_proj ? c2(s.red[3 + 2 * tid], s.red[4 + 2 * tid])
-                                       : (chk(a.dbg, 12, a.cidx[tid], a.n) ? Vec<R>::wide(__ldcg(a.r + a.cidx[tid])) : c2(0, 0));
+                                       : (chk(a.dbg, 12, s_cidx[tid], a.n) ? Vec<R>::wide(__ldcg(a.r + s_cidx[tid])) : c2(0, 0));
         }
         __syncthreads();
         if (s.bnorm == 0.0) {                 // b = 0: x = 0 solves every shift
-            if (owns) { a.S.frozen[k_own] = 1; a.S.resid[k_own] = 0.0; }
+            if (owns) { S.frozen[ko] = 1; S.resid[ko] = 0.0; }
             status = SCOCG_OK;
             done = true;
         }
     }
 
     // ------------------------------------------------------------ iterations
+    int it = s.n;                             // seed iteration, every thread's own copy
+    // scalars of the next reductions that depend on the last iteration only,
+    // by warp 1 while the other warps apply H
+    auto prepare_scalars = [&]() {
+        const double2 ir = warp_cdiv(c2(1, 0), s.rho);
+        const double2 gr = warp_cdiv(s.beta_prev, s.alpha_prev);
+        if (lane == 0) { s.inv_rho = ir; s.t2_ratio = gr; }
+    };
     bool skip_a = kResume;                    // the continued solve's first phase A ran before it stopped
     while (!done) {
         SCOCG_TRACE(1);
@@ -470,79 +758,104 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
         // ---- phase A: q_n = (z_s - H) r_n + beta_{n-1} q_{n-1}; partial r_n^T q_n
         // (with a deferred phase C of iteration n-1 in warp 0)
         if (!skip_a) {
-            const V zs = s_vs[0];
-            const V bp = s_vs[1];
             AT rq[2] = {};
+            // (z_s and beta are read from shared memory where they are used: kept
+            // in registers across the apply they would be spilled)
+
             const bool c_here = pending;           // uniform over the grid
             if (c_here && warp == 0) {
                 int act = 0, bad = 0;
-                if (owns && !a.S.frozen[k_own]) shift_update(a, k_own, s_c, M, tol2, act, bad);
-                act = __popc(__ballot_sync(0xffffffffu, act));
-                bad = __any_sync(0xffffffffu, bad);
+                if (own_wide) {
+                    shift_update_warp(s_own, nown, s_c, M, a.tol, tol2, act, bad);
+                } else {
+                    if (owns && !state().frozen[ko]) update_own(act, bad);
+                    act = __popc(__ballot_sync(0xffffffffu, act));
+                    bad = __any_sync(0xffffffffu, bad);
+                }
                 if (lane == 0) { s_flag[0] = act; s_flag[1] = bad; }
             }
+            if (warp == 1) prepare_scalars();
             // all warps apply H; with a deferred phase C the unit order is
-            // rotated so that warp 0 takes the last place in each round and,
-            // when the rounds do not come out even, one unit fewer
-            const int wi = c_here ? (warp + kWarps - 1) % kWarps : warp;
-            const int64_t a_first = Apply::kMap == kMapStrided ? (int64_t)cta + (int64_t)G * wi : ubeg + wi;
+            // rotated so that warps 0 and 1 take the last places in each round
+            // and, when the rounds do not come out even, one unit fewer
+            const int wi = c_here ? rotated_place(warp) : warp;
             if constexpr (HasTwoPass<Apply>::value) {
                 // two passes over the units in two orders, a grid barrier between
-                for (int64_t u = a_first; u < u_end; u += u_step) ap.pass1(u, lane, zs, bp, (const V*)a.r, a.q);
+                for (int lu = wi; lu < sh.nloc; lu += kWarps) ap.pass1(sh.unit(lu), lane, s_vs[0], s_vs[1], (const V*)a.r, a.q);
                 if (!grid_barrier(a.sync, epoch)) return;
-                for (int64_t u = a_first; u < u_end; u += u_step) {
+                for (int lu = wi; lu < sh.nloc; lu += kWarps) {
                     int64_t row;
                     V qn;
-                    if (ap.pass2(u, lane, (const V*)a.r, a.q, row, qn)) acc_bil(rq[0], rq[1], a.r[row], qn);
+                    if (ap.pass2(sh.unit(lu), lane, (const V*)a.r, a.q, row, qn)) acc_bil(rq[0], rq[1], a.r[row], qn);
                 }
             } else {
-                for (int64_t u = a_first; u < u_end; u += u_step) {
+                for (int lu = wi; lu < sh.nloc; lu += kWarps) {
                     int64_t row;
                     V w;
-                    if (ap(u, lane, zs, (const V*)a.r, row, w)) {
-                        const V qn = vcfma(bp, a.q[row], w);
-                        a.q[row] = qn;
+                    if (ap(sh.unit(lu), lane, s_vs[0], (const V*)a.r, row, w)) {
+                        const int t = sh.place(lu, lane);
+                        const V qn = vcfma(s_vs[1], sh.get(t, row), w);
+                        sh.put(t, row, qn);
                         acc_bil(rq[0], rq[1], a.r[row], qn);
                     }
                 }
             }
-            block_partials<2>(rq, s.scratch, a.partA + cta, G, wi, 2, nwA);
+            ++red_no;
+            // (only thread 0's tag is read, and it has set the counts itself)
+            const unsigned long long tag = pkt && tid == 0 ? packet_tag(red_no, s_flag[0], s_flag[1]) : red_no;
+            block_partials<2>(rq, s_scratch,
+                              PartialOut{a.partA + cta, pkt ? a.pk + cta : nullptr, G, tag,
+                                         a.debug_inject == 1 && cta == 0 && it == 3}, wi, 2, nwA);
             pending = false;
-            if (tid == 64) a.partA[2 * G + cta] = pack_counts(s_flag[0], s_flag[1]);
+            if (!pkt && tid == 64) a.partA[2 * G + cta] = pack_counts(s_flag[0], s_flag[1]);
+        } else if (warp == 1) {
+            prepare_scalars();
         }
         skip_a = false;
         SCOCG_TRACE(2);
         SCOCG_MARK(0);
-        if (!grid_barrier(a.sync, epoch, a.debug_inject == 1 && cta == 0 && s.n == 3)) return;
-        SCOCG_TRACE(3);
-        SCOCG_MARK(1);
-        if (warp == 2) {
-            int act, bad;
-            sum_counts(a.partA + 2 * G, G, act, bad);
-            if (lane == 0) { s_flag[5] = act; s_flag[6] = bad; }
-        }
-        grid_sum_vm1(a.partA, 2, s.red, G);
-        if (tid == 0) {
-            const double2 rq = c2(s.red[0], s.red[1]);
-            const int active = s.n == 0 ? a.K : s_flag[5];
-            int st = kGoOn;
-            if (s.n > 0 && s_flag[6] != 0) st = SCOCG_ERR_BREAKDOWN;
-            else if (active == 0) st = SCOCG_OK;
-            else if (s.n >= a.max_iter) st = SCOCG_NOT_CONVERGED;
-            else if (cabs2(s.rho) == 0.0 || cabs2(rq) == 0.0 || !cfinite(rq)) st = SCOCG_ERR_BREAKDOWN;
-            else {
-                s.alpha = cdiv(s.rho, rq);
-                if (a.debug_inject == 2 && s.n == 3) s.alpha = c2(__longlong_as_double(0x7ff8000000000000ll), 0);
-                if (!cfinite(s.alpha)) st = SCOCG_ERR_BREAKDOWN;
-                s_vs[2] = Vec<R>::make(s.alpha);
-                s.shift_iters += active;
+        if (pkt) {
+            if (!packet_sums(a.sync, a.pk, G, 2, red_no, s.red, s_flag + 5)) return;
+            SCOCG_TRACE(3);
+            SCOCG_MARK(1);
+        } else {
+            if (!grid_barrier(a.sync, epoch, a.debug_inject == 1 && cta == 0 && it == 3)) return;
+            SCOCG_TRACE(3);
+            SCOCG_MARK(1);
+            if (warp == 2) {
+                int act, bad;
+                sum_counts(a.partA + 2 * G, G, act, bad);
+                if (lane == 0) { s_flag[5] = act; s_flag[6] = bad; }
             }
+            grid_sum_vm1(a.partA, 2, s.red, G);
+        }
+        // warp 0 forms alpha while thread 32 makes the other checks
+        if (warp == 0) {
+            double2 al = warp_cdiv(s.rho, c2(s.red[0], s.red[1]));
+            if (a.debug_inject == 2 && it == 3) al = c2(__longlong_as_double(0x7ff8000000000000ll), 0);
+            if (lane == 0) {
+                s.alpha = al;
+                s_vs[2] = Vec<R>::make(al);
+                s_flag[3] = cfinite(al);
+            }
+        } else if (tid == 32) {
+            const double2 rq = c2(s.red[0], s.red[1]);
+            const int active = it == 0 ? a.K : s_flag[5];
+            int st = kGoOn;
+            if (it > 0 && s_flag[6] != 0) st = SCOCG_ERR_BREAKDOWN;
+            else if (active == 0) st = SCOCG_OK;
+            else if (it >= a.max_iter) st = SCOCG_NOT_CONVERGED;
+            else if (cabs2(s.rho) == 0.0 || cabs2(rq) == 0.0 || !cfinite(rq)) st = SCOCG_ERR_BREAKDOWN;
+            if (st == kGoOn) s.shift_iters += active;
             s.active = active;
             s_flag[2] = st;
         }
         __syncthreads();
         SCOCG_MARK(6);
-        if (s_flag[2] != kGoOn) { status = s_flag[2]; break; }
+        if (s_flag[2] != kGoOn || !s_flag[3]) {
+            status = s_flag[2] != kGoOn ? s_flag[2] : (int)SCOCG_ERR_BREAKDOWN;
+            break;
+        }
 
         // ---- full-vector mode: this iteration's shift scalars for all shifts
         // (every CTA computes them, with the same arithmetic as phase C).  The
@@ -567,7 +880,7 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
                     const double2 pn = cadd(cmul(cadd(c2(1, 0), cmul(s.alpha, __ldcg(a.S.sigma + k))), pc),
                                             cmul(t2, csub(pc, pp)));
                     const double2 in = crecip(pn);
-                    const double2 t = s.n == 0 ? c2(1, 0) : s_t[k];
+                    const double2 t = it == 0 ? c2(1, 0) : s_t[k];
                     s_cp[k] = cmul(cmul(cmul(cmul(ratio, ratio), s.beta_prev), pc), t);
                     s_cx[k] = cmul(cmul(cmul(pc, in), s.alpha), ic);
                     s_t[k] = ic;
@@ -577,11 +890,11 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
                 // Warps take 32-row chunks of the CTA's rows; when there are
                 // fewer chunks than warps, several warps share a chunk's shifts.
                 // Four shifts' vectors are in flight per warp.
-                const int nch = (int)((rend - rbeg + 31) >> 5), nact = s_nact;
+                const int nch = (sh.nrow + 31) >> 5, nact = s_nact;
                 const int share = nch < kWarps ? kWarps / max(nch, 1) : 1;
                 for (int c = warp / share; c < nch; c += kWarps / share) {
-                    const int64_t i = rbeg + 32 * c + lane;
-                    if (i >= rend) continue;
+                    if (32 * c + lane >= sh.nrow) continue;
+                    const int64_t i = sh.row(32 * c + lane);
                     const double2 ri = a.r[i];
                     constexpr int kU = 4;
                     for (int j0 = (warp % share) * kU; j0 < nact; j0 += share * kU) {
@@ -615,20 +928,27 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
             if (plain) {
                 // one row ahead: the next row's loads are in flight while this
                 // row is updated and stored (same rows, same order per thread)
-                int64_t i = rbeg + tid;
                 V ro = vzero<V>(), qo = vzero<V>(), co = vzero<V>();
-                if (i < rend) { ro = a.r[i]; qo = a.q[i]; if (a.cvec) co = a.cvec[i]; }
-                for (; i < rend; i += kBlock) {
-                    const int64_t inx = i + kBlock;
+                if (tid < sh.nrow) {
+                    const int64_t i = sh.row(tid);
+                    ro = a.r[i]; qo = sh.get(tid, i);
+                    if (a.cvec) co = a.cvec[i];
+                }
+                for (int t = tid; t < sh.nrow; t += kBlock) {
                     V r1 = vzero<V>(), q1 = vzero<V>(), c1 = vzero<V>();
-                    if (inx < rend) { r1 = a.r[inx]; q1 = a.q[inx]; if (a.cvec) c1 = a.cvec[inx]; }
+                    if (t + kBlock < sh.nrow) {
+                        const int64_t i1 = sh.row(t + kBlock);
+                        r1 = a.r[i1]; q1 = sh.get(t + kBlock, i1);
+                        if (a.cvec) c1 = a.cvec[i1];
+                    }
                     const V rn = r_update(ro, al, qo);
-                    a.r[i] = rn;
+                    a.r[sh.row(t)] = rn;
                     acc_r<R>(acc, rn, a.cvec ? &co : nullptr);
                     ro = r1; qo = q1; co = c1;
                 }
             }
-            for (int64_t i = rbeg + tid; !plain && i < rend; i += kBlock) {
+            for (int t = tid; !plain && t < sh.nrow; t += kBlock) {
+                const int64_t i = sh.row(t);
                 const V ro = a.r[i];
                 if constexpr (kMixed) {
                     if (track_x) {
@@ -646,35 +966,46 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
                         a.x_lo[i] = lo;
                     }
                 }
-                const V rn = r_update(ro, al, a.q[i]);
+                const V rn = r_update(ro, al, sh.get(t, i));
                 a.r[i] = rn;
                 acc_r<R>(acc, rn, a.cvec ? a.cvec + i : nullptr);
             }
             __syncthreads();
-            finish_r_partials(a, acc, rbeg, rend, s, myB, G);
+            ++red_no;
+            finish_r_partials(a, acc, sh, s_scratch,
+                              PartialOut{myB, pkt ? a.pk + 2 * G + cta : nullptr, G, red_no, false});
         }
         SCOCG_TRACE(4);
         SCOCG_MARK(2);
-        if (!grid_barrier(a.sync, epoch)) return;
-        SCOCG_TRACE(5);
-        SCOCG_MARK(3);
-        grid_sum_vm1(a.partB, nred, s.red, G);
+        if (pkt) {
+            if (!packet_sums(a.sync, a.pk + 2 * G, G, nred, red_no, s.red, s_flag + 5)) return;
+        } else {
+            if (!grid_barrier(a.sync, epoch)) return;
+            SCOCG_TRACE(5);
+            SCOCG_MARK(3);
+            grid_sum_vm1(a.partB, nred, s.red, G);
+        }
         SCOCG_MARK(5);
         // the scalars of this iteration: independent FP64 chains run in three
         // warps at once
         if (tid < M) {
             s.cr_next[tid] = dense_proj ? c2(s.red[3 + 2 * tid], s.red[4 + 2 * tid])
-                                        : (chk(a.dbg, 12, a.cidx[tid], a.n) ? Vec<R>::wide(__ldcg(a.r + a.cidx[tid])) : c2(0, 0));
+                                        : (chk(a.dbg, 12, s_cidx[tid], a.n) ? Vec<R>::wide(__ldcg(a.r + s_cidx[tid])) : c2(0, 0));
             s_c.cr[tid] = s.cr_cur[tid];
+            s.cr_cur[tid] = s.cr_next[tid];
         }
-        if (tid == 0) {
-            s.t2 = cdiv(cmul(s.alpha, s.beta_prev), s.alpha_prev);
-            s_c.alpha = s.alpha; s_c.beta_prev = s.beta_prev; s_c.t2 = s.t2; s_c.n = s.n;
+        if (tid == 96) {
+            s_c.t2 = cmul(s.alpha, s.t2_ratio);
+            s_c.alpha = s.alpha; s_c.beta_prev = s.beta_prev; s_c.n = it;
         } else if (tid == 32) {
             s_c.rn_b2 = s.red[2] * s.inv_b2;
             s_flag[4] = a.tol > 0.0 && s_c.rn_b2 <= tol2;    // the seed (pi = 1) has converged
-        } else if (tid == 64) {
-            s.beta_next = cdiv(c2(s.red[0], s.red[1]), s.rho);
+        } else if (warp == 2) {
+            const double2 be = warp_quot(c2(s.red[0], s.red[1]), s.rho, s.inv_rho);
+            if (lane == 0) {
+                s.beta_next = be;
+                s_vs[1] = Vec<R>::make(be);
+            }
         }
         __syncthreads();
 
@@ -685,22 +1016,23 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
         const bool defer = defer_ok && !seed_conv;
         if (!defer) {
             int my_active = 0, my_bad = 0;
-            if (owns && !a.S.frozen[k_own]) shift_update(a, k_own, s_c, M, tol2, my_active, my_bad);
+            if (owns && !state().frozen[ko]) update_own(my_active, my_bad);
             const int cnt_active = __syncthreads_count(my_active);
             const int any_bad = __syncthreads_or(my_bad);
             if (tid == 0) { s_flag[0] = cnt_active; s_flag[1] = any_bad; }
         }
         pending = defer;
-        if (tid == 0) {
+        ++it;
+        // (read next by warp 1, and after further CTA synchronisations by others)
+        if (tid == 32) {
             s.beta_prev = s.beta_next;
-            s_vs[1] = Vec<R>::make(s.beta_prev);
             s.alpha_prev = s.alpha;
             s.rho_prev = s.rho;
             s.rho = c2(s.red[0], s.red[1]);
-            s.n += 1;
+            s.n = it;
         }
-        if (tid < M) s.cr_cur[tid] = s.cr_next[tid];
-        __syncthreads();
+        if (warp == 1) __syncwarp();
+        if (kMixed || seed_conv) __syncthreads();
 
         // ---- seed switching (Sec. III.C) once the seed has converged
         SCOCG_TRACE(6);
@@ -710,7 +1042,8 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
             // local candidate: the unconverged shift with the smallest |pi| (largest residual)
             double best = INFINITY;
             int arg = 0x7fffffff;
-            if (owns && !a.S.frozen[k_own]) { best = -cabs2(a.S.inv_cur[k_own]); arg = k_own; }
+            const ShiftState S = state();
+            if (owns && !S.frozen[ko]) { best = -cabs2(S.inv_cur[ko]); arg = k_own; }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
                 const double ob = __shfl_xor_sync(0xffffffffu, best, o);
@@ -727,7 +1060,8 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
                 double* pc = a.partC + (size_t)cta * kPartC;
                 pc[0] = (double)s_flag[0]; pc[1] = best; pc[2] = (double)arg; pc[3] = (double)s_flag[1];
                 if (arg < a.K && chk(a.dbg, 10, arg, a.K)) {
-                    const double2 pp = a.S.pi_prev[arg], pq = a.S.pi_cur[arg], ak = a.S.alpha_k[arg];
+                    const int ka = own_sm ? (arg - cta) / G : arg;
+                    const double2 pp = S.pi_prev[ka], pq = S.pi_cur[ka], ak = S.alpha_k[ka];
                     pc[4] = pp.x; pc[5] = pp.y; pc[6] = pq.x; pc[7] = pq.y; pc[8] = ak.x; pc[9] = ak.y;
                 }
             }
@@ -768,22 +1102,22 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
             const double2 ca = cdiv(csub(cdiv(c2(1, 0), pin), inv1), alpha_s2);   // times r_{n+1}
             const double2 cb = cdiv(cdiv(s.alpha_prev, pin), alpha_s2);           // times q_n
             const V v_inv1 = Vec<R>::make(inv1), v_ca = Vec<R>::make(ca), v_cb = Vec<R>::make(cb);
-            for (int64_t i = rbeg + tid; i < rend; i += kBlock) {
-                const V ri = a.r[i], qi = a.q[i];
-                a.q[i] = vcfma(v_cb, qi, vcfma(v_ca, ri, vzero<V>()));
+            for (int t = tid; t < sh.nrow; t += kBlock) {
+                const int64_t i = sh.row(t);
+                const V ri = a.r[i], qi = sh.get(t, i);
+                sh.put(t, i, vcfma(v_cb, qi, vcfma(v_ca, ri, vzero<V>())));
                 a.r[i] = vcfma(v_inv1, ri, vzero<V>());
             }
             SCOCG_TRACE(11);
             if (owns && chk(a.dbg, 13, s2, a.K)) {
-                const int k = k_own;
-                if (k == s2) {
-                    a.S.pi_prev[k] = c2(1, 0); a.S.pi_cur[k] = c2(1, 0); a.S.inv_cur[k] = c2(1, 0);
+                if (k_own == s2) {
+                    S.pi_prev[ko] = c2(1, 0); S.pi_cur[ko] = c2(1, 0); S.inv_cur[ko] = c2(1, 0);
                 } else {
-                    a.S.pi_prev[k] = cdiv(a.S.pi_prev[k], pin);
-                    a.S.pi_cur[k] = cdiv(a.S.pi_cur[k], pin1);
-                    a.S.inv_cur[k] = cmul(a.S.inv_cur[k], pin1);
+                    S.pi_prev[ko] = cdiv(S.pi_prev[ko], pin);
+                    S.pi_cur[ko] = cdiv(S.pi_cur[ko], pin1);
+                    S.inv_cur[ko] = cmul(S.inv_cur[ko], pin1);
                 }
-                a.S.sigma[k] = csub(a.z[k], a.z[s2]);
+                S.sigma[ko] = csub(a.z[k_own], a.z[s2]);
             }
             __syncthreads();
             if (tid == 0) {
@@ -806,23 +1140,24 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
 
         // ---- MIXED: FP64 true-residual replacement r_{n+1} = b - (z_s - H) x_{n+1}
         if constexpr (kMixed) {
-            if (s.replace_on && s.n % a.replace_every == 0) {
-                for (int64_t i = rbeg + tid; i < rend; i += kBlock) {
+            if (s.replace_on && it % a.replace_every == 0) {
+                for (int t = tid; t < sh.nrow; t += kBlock) {
+                    const int64_t i = sh.row(t);
                     const V hi = a.x_hi[i], lo = a.x_lo[i];
                     a.xd[i] = c2((double)hi.x + (double)lo.x, (double)hi.y + (double)lo.y);
                 }
                 if (!grid_barrier(a.sync, epoch)) return;
                 const double2 zs = s.zs;
-                for (int64_t u = u_first; u < u_end; u += u_step) {
+                for (int lu = warp; lu < sh.nloc; lu += kWarps) {
                     int64_t row;
                     double2 w;
-                    if (ap(u, lane, zs, (const double2*)a.xd, row, w)) {
+                    if (ap(sh.unit(lu), lane, zs, (const double2*)a.xd, row, w)) {
                         const double2 bi = a.b[row];
                         a.r[row] = Vec<R>::make(c2(bi.x - w.x, bi.y - w.y));
                     }
                 }
                 if (!grid_barrier(a.sync, epoch)) return;
-                r_partials(a, rbeg, rend, s, myB, G);
+                r_partials(a, sh, s_scratch, outB);
                 if (!grid_barrier(a.sync, epoch)) return;
                 grid_sum_vm1(a.partB, nred, s.red, G);
                 if (tid == 0) {
@@ -833,7 +1168,7 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
                 }
                 if (tid < M) {
                     s.cr_cur[tid] = dense_proj ? c2(s.red[3 + 2 * tid], s.red[4 + 2 * tid])
-                                               : (chk(a.dbg, 12, a.cidx[tid], a.n) ? Vec<R>::wide(__ldcg(a.r + a.cidx[tid])) : c2(0, 0));
+                                               : (chk(a.dbg, 12, s_cidx[tid], a.n) ? Vec<R>::wide(__ldcg(a.r + s_cidx[tid])) : c2(0, 0));
                 }
                 __syncthreads();
             }
@@ -842,8 +1177,21 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
 
     // ------------------------------------------------------------ outputs
     SCOCG_TRACE(20);
+    // what a continuation starts from
+    if (sh.on && a.rstate && status == SCOCG_NOT_CONVERGED)
+        for (int t = tid; t < sh.nrow; t += kBlock) a.q[sh.row(t)] = sh.q_s[t];
+    const ShiftState S = state();
     if (owns) {
-        for (int m = 0; m < M; ++m) a.G[(size_t)m * a.K + k_own] = a.S.X[(size_t)k_own * M + m];
+        for (int m = 0; m < M; ++m) a.G[(size_t)m * a.K + k_own] = S.X[(size_t)ko * M + m];
+        if (own_sm) {
+            a.S.pi_prev[k_own] = S.pi_prev[ko]; a.S.pi_cur[k_own] = S.pi_cur[ko]; a.S.inv_cur[k_own] = S.inv_cur[ko];
+            a.S.sigma[k_own] = S.sigma[ko]; a.S.alpha_k[k_own] = S.alpha_k[ko];
+            for (int m = 0; m < M; ++m) {
+                a.S.P[(size_t)k_own * M + m] = S.P[ko * M + m];
+                a.S.X[(size_t)k_own * M + m] = S.X[ko * M + m];
+            }
+            a.S.frozen[k_own] = S.frozen[ko]; a.S.iters[k_own] = S.iters[ko]; a.S.resid[k_own] = S.resid[ko];
+        }
     }
     if (cta == 0 && tid == 0) {
         // the stopping apply took the deferred shift update (and rotated its
