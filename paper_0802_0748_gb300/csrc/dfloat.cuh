@@ -26,7 +26,7 @@ __device__ __forceinline__ void fast_two_sum(float a, float b, float& s, float& 
     e = b - (s - a);
 }
 __device__ __forceinline__ void two_prod(float a, float b, float& p, float& e) {
-    p = a * b;
+    p = __fmul_rn(a, b);
     e = fmaf(a, b, -p);
 }
 
@@ -58,15 +58,6 @@ __device__ __forceinline__ void df_acc_prod(dfs& acc, dfs a, dfs b) {
     acc.hi = s;
     acc.lo += t + e;
 }
-// acc += v * x for a float v and a DF x (the H apply)
-__device__ __forceinline__ void df_acc_fx(dfs& acc, float v, float xhi, float xlo) {
-    float p, e, s, t;
-    two_prod(v, xhi, p, e);
-    e = fmaf(v, xlo, e);
-    two_sum(acc.hi, p, s, t);
-    acc.hi = s;
-    acc.lo += t + e;
-}
 
 __device__ __forceinline__ dfs cre(float4 v) { return dfs{v.x, v.z}; }
 __device__ __forceinline__ dfs cim(float4 v) { return dfs{v.y, v.w}; }
@@ -81,6 +72,13 @@ __device__ __forceinline__ float2 pk_add(float2 a, float2 b) { return __fadd2_rn
 __device__ __forceinline__ float2 pk_sub(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
 __device__ __forceinline__ float2 pk_mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 pk_fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+// a rounded product that an addition follows: the assembler fuses a paired
+// multiply whose only use is a paired addition into one FMA (the sum's error
+// then loses the product's own rounding: 1.6e-8 instead of 3e-14 on 28-term
+// sums), which it does not do with the scalar multiply
+__device__ __forceinline__ float2 pk_mul_rn(float2 a, float2 b) {
+    return make_float2(__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y));
+}
 __device__ __forceinline__ float2 pk_neg(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.x, v.y); }
 __device__ __forceinline__ float2 lo2(float4 v) { return make_float2(v.z, v.w); }
@@ -99,7 +97,10 @@ __device__ __forceinline__ void pk_norm(float2& hi, float2& lo) {
     hi = s;
 }
 // (ah, al) += (xh + xl) * (yh + yl) lane by lane, the product exact to DF and
-// the sum by TwoSum, without renormalising the accumulator
+// the sum by TwoSum, without renormalising the accumulator.  (Folding the
+// product's remainder into the TwoSum as below saves one instruction here but
+// rounds the low part twice more: the 64^3 x 4 solve at Im z = 1e-3 then took
+// more than 400,000 iterations instead of 120,000.)
 __device__ __forceinline__ void pk_acc_prod(float2& ah, float2& al, float2 xh, float2 xl, float2 yh, float2 yl) {
     const float2 p = pk_mul(xh, yh);
     float2 e = pk_fma(xh, yh, pk_neg(p));
@@ -108,6 +109,20 @@ __device__ __forceinline__ void pk_acc_prod(float2& ah, float2& al, float2 xh, f
     pk_two_sum(ah, p, s, t);
     ah = s;
     al = pk_add(al, pk_add(t, e));
+}
+// (ah, al) += v * (xh + xl) for an FP32 v, the apply's step.  With p the rounded
+// product and s = ah + p by TwoSum (bb = s - ah), the two exact remainders
+// (v xh - p) + (p - bb) are one fused operation, v xh - bb, rounded once: 21
+// cycles of a scheduler's FP32 pipe per warp (a paired add holds it two cycles,
+// a paired FMA 2.4) instead of 26 with TwoProd and TwoSum one after the other,
+// at the same error of a 28-term sum (rms 2.74e-15 against 2.70e-15 of the terms'
+// magnitude).  The apply's 28 steps per row are what that pipe spends most of its
+// time on.
+__device__ __forceinline__ void pk_acc_fx2(float2& ah, float2& al, float2 v, float2 xh, float2 xl) {
+    const float2 s = pk_add(ah, pk_mul_rn(v, xh)), bb = pk_sub(s, ah);
+    const float2 u = pk_add(pk_sub(ah, pk_sub(s, bb)), pk_fma(v, xh, pk_neg(bb)));
+    ah = s;
+    al = pk_add(al, pk_fma(v, xl, u));
 }
 
 // complex a * b + c: (re, im) += (a.re, a.re) (b.re, b.im) + (-a.im, a.im) (b.im, b.re)
@@ -129,15 +144,9 @@ __device__ __forceinline__ float4 vsub(float4 a, float4 b) {
 }
 // acc += v * x (real float v); acc is kept unnormalised until the apply ends
 __device__ __forceinline__ void cfma_r(float4& acc, float v, float4 x) {
-    const float2 vv = make_float2(v, v);
     float2 h = hi2(acc), l = lo2(acc);
-    const float2 xh = hi2(x);
-    const float2 p = pk_mul(vv, xh);
-    float2 e = pk_fma(vv, xh, pk_neg(p));
-    e = pk_fma(vv, lo2(x), e);
-    float2 s, t;
-    pk_two_sum(h, p, s, t);
-    acc = pk4(s, pk_add(l, pk_add(t, e)));
+    pk_acc_fx2(h, l, make_float2(v, v), hi2(x), lo2(x));
+    acc = pk4(h, l);
 }
 // sum of two unnormalised compensated complex accumulators, normalised
 __device__ __forceinline__ float4 vadd_acc(float4 a, float4 b) {

@@ -442,14 +442,7 @@ __global__ void __launch_bounds__(kVecBlock) k_krylov_block(KrylovBlockArgs a) {
 // the step scalars stay FP64.  Two rows of a block row share each paired
 // FP32 instruction of the apply.
 __device__ __forceinline__ void pk_acc_fx(float2& ah, float2& al, float2 v, float xh, float xl) {
-    const float2 xh2 = make_float2(xh, xh);
-    const float2 p = pk_mul(v, xh2);
-    float2 e = pk_fma(v, xh2, pk_neg(p));
-    e = pk_fma(v, make_float2(xl, xl), e);
-    float2 s, t;
-    pk_two_sum(ah, p, s, t);
-    ah = s;
-    al = pk_add(al, pk_add(t, e));
+    pk_acc_fx2(ah, al, v, make_float2(xh, xh), make_float2(xl, xl));
 }
 __device__ __forceinline__ dfs df_of(double v) {
     const float hi = (float)v;
