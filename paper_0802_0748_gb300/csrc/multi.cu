@@ -140,7 +140,7 @@ int run_multi(int nsys, const scocg_handle* hs, const scocg_c128* const* shifts,
             const int rpu = rows_per_unit(L.kind);
             units[s] = (hs[s]->n + rpu - 1) / rpu;
             gmin[s] = std::max<int64_t>(1, (nshift[s] + kBlock - 1) / kBlock);
-            gmax[s] = std::max<int64_t>(gmin[s], (units[s] + kWarps - 1) / kWarps);
+            gmax[s] = std::max<int64_t>(gmin[s], grid_want(units[s], prec == SCOCG_FP64, h0->num_sms, maxco));
             tot_units += units[s];
             need += gmin[s];
         }

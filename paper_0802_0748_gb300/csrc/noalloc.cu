@@ -154,7 +154,7 @@ extern "C" int scocg_solve_csr_noalloc(int64_t n, int64_t nnz, const int32_t* ro
     const int rpu = 32 / lpr;
     const int64_t nunits = (n + rpu - 1) / rpu;
     const int K = nshift, M = nproj;
-    int64_t want = std::max<int64_t>((nunits + kWarps - 1) / kWarps, (K + kBlock - 1) / kBlock);
+    int64_t want = std::max<int64_t>(grid_want(nunits, true, sms, (int64_t)occ * sms), (K + kBlock - 1) / kBlock);
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)occ * sms));
     if ((int64_t)grid * kBlock < K) return SCOCG_ERR_TOO_LARGE;
     const int strideB = 3 + 2 * M + 1;

@@ -23,6 +23,8 @@
 // every `replace_every` iterations replaces r by the FP64 true residual
 // b - A x (reliable update).
 #pragma once
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace scocg {
@@ -31,7 +33,7 @@ constexpr int kMaxProjB = 4;   // unit projections per right-hand side of a bloc
 #ifndef SCOCG_BSR4_GROUP
 #define SCOCG_BSR4_GROUP 4     // slots of the blocked apply whose loads are issued together
 #endif
-constexpr int kPktCtas = 64, kPktVals = 7;
+constexpr int kPktCtas = 32, kPktVals = 7;
 constexpr int kPartC = 10;   // active, best |pi|, arg, bad, pi_prev, pi_cur, alpha_k of arg
 
 struct ShiftState {          // device arrays, [K] or [K][M]
@@ -396,6 +398,20 @@ inline size_t q_smem_bytes(int64_t nunits, int rows_per_unit, int grid) {
 template <typename R>
 inline size_t solve_smem(const SolveArgs<R>& a, int grid) {
     return full_smem(a.Xf ? a.K : 0) + (a.q_smem ? q_smem_bytes<R>(a.nunits, a.rows_per_unit, grid) : 0);
+}
+// CTAs that a solve of `units` units of rows asks for (the caller clamps it to
+// what can be co-resident, maxco).  An iteration has about 10 us of serial work
+// whatever the grid, so CTAs are added only while they shorten the phases: a
+// complex128 unit occupies a scheduler's FP64 pipe ~4 us, so four units (one per
+// scheduler) make a CTA; eight FP32 units do.  16^3 x 4 FP64 (512 units): 23.6 us
+// per iteration at 32 CTAs, 13.7 at 128; 22^3 x 4 FP64: 24.4 at 84, 17.9 at 152;
+// 8^3 x 4 (64 units) FP64 11.6 at 16, 12.9 at 64, compensated 11.1 at 8, 13.7 at
+// 32.  One CTA per SM serves up to 24 units per SM (30^3 x 4 compensated, 22 per
+// SM: 20.1 at 152, 21.0 at 211, 19.9 at 304), above that every SM takes all it can.
+inline int64_t grid_want(int64_t units, bool fp64, int num_sms, int64_t maxco) {
+    const int64_t per = fp64 ? 4 : 8;
+    if (units > 24LL * num_sms) return maxco;
+    return std::max<int64_t>(std::min<int64_t>(units, 16), std::min<int64_t>((units + per - 1) / per, num_sms));
 }
 // q is kept in shared memory while the CTAs of an SM hold at most this much of
 // it: the rest of the SM's 256 KB is the L1 that the gathers of the apply use.

@@ -24,7 +24,7 @@ template <> __device__ __forceinline__ double unpark<dfs>(const double* slot) {
 
 // Where a CTA's partial sums of one reduction go: value j to part[j * G] (read
 // after a grid barrier), or, with pk set, to packet pk[j * G] = {value, tag}
-// that the other CTAs wait for directly (grids up to kPktCtas).
+// that the other CTAs wait for directly (grids up to kPktCtas = 32).
 struct PartialOut {
     double* part;
     ulonglong2* pk;
@@ -370,27 +370,25 @@ __device__ __forceinline__ unsigned long long packet_tag(unsigned no, int active
     return ((unsigned long long)((unsigned)active | (bad ? 0x80000000u : 0u)) << 32) | no;
 }
 
-// Waits for nv packets of each of the G CTAs (warp j < nv for packet j, two
-// CTAs per lane) and leaves their sums, the same in every CTA, in out[0..nv)
+// Waits for nv packets of each of the G <= 32 CTAs (warp j < nv for packet j,
+// lane c for CTA c) and leaves their sums, the same in every CTA, in out[0..nv)
 // and the counts of packet 0 in counts[0..1] (counts[2]: a wait was given up).  One round trip through L2
 // instead of the barrier's arrival, its poll and then the loads of the
-// partials (32 CTAs: 1.1 us against 1.25 + 0.6).  A packet is rewritten only
+// partials (32 CTAs: 1.1 us against 1.25 + 0.6; at 64 CTAs the packets' all-to-all
+// traffic makes it the slower one).  A packet is rewritten only
 // after a later reduction that every CTA takes part in.  The wait is bounded
 // like the grid barrier's; false ends the solve.
 __device__ __forceinline__ bool packet_sums(const GridSync& g, const ulonglong2* pk, int G, int nv, unsigned no,
                                             double* out, int* counts) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (warp < nv) {
-        double v[2] = {0.0, 0.0};
+        double v = 0.0;
         unsigned aux = 0u, any = 0u;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int c = lane + 32 * h;
-            if (c >= G) break;
+        if (lane < G) {
             unsigned long long tag = 0;
             uint64_t t0 = 0;
             for (unsigned turn = 1;; ++turn) {
-                v[h] = ld_packet(pk + (size_t)warp * G + c, tag);
+                v = ld_packet(pk + (size_t)warp * G + lane, tag);
                 if ((unsigned)tag == no) break;
                 if (turn & 63u) continue;
                 const uint64_t t = globaltimer_ns();
@@ -402,12 +400,12 @@ __device__ __forceinline__ bool packet_sums(const GridSync& g, const ulonglong2*
                     break;
                 }
             }
-            aux += (unsigned)(tag >> 32) & 0x7fffffffu;
-            any |= (unsigned)(tag >> 63);
+            aux = (unsigned)(tag >> 32) & 0x7fffffffu;
+            any = (unsigned)(tag >> 63);
         }
         __syncwarp();
         fence_acq_rel();   // the CTA's later loads see the writes before the packets
-        const double t = warp_sum(G > 32 ? v[0] + v[1] : v[0]);
+        const double t = warp_sum(v);
         if (lane == 0) out[warp] = t;
         if (warp == 0) {
             aux = __reduce_add_sync(0xffffffffu, aux);
