@@ -527,22 +527,33 @@ __global__ void __launch_bounds__(kVecBlock) k_krylov_block_df(KrylovBlockDfArgs
             const int64_t u = B >> 3;
             const int br = (int)(B & 7);
             const int s0 = a.unit_off[u], s1 = a.unit_off[u + 1];
-            for (int sl = s0; sl < s1; ++sl) {
-                const int cb = ld_stream(a.bcol + (size_t)sl * 8 + br);
-                if (cb < 0) continue;
-                float2 xv[4];
+            // kPre slots at a time: their column-block indices, then their
+            // gathers of x, are in flight together (a padded or absent slot
+            // reads block 0 and is skipped)
+            constexpr int kPre = 4;
+            for (int g0 = s0; g0 < s1; g0 += kPre) {
+                int cb[kPre];
+                float2 xv[kPre][4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) xv[q] = wprev[((size_t)cb * 4 + q) * T + cl];
-                const float4* hb = reinterpret_cast<const float4*>(a.bval + ((size_t)sl * 8 + br) * 16);
-                const float4 r0 = ld_stream(hb), r1 = ld_stream(hb + 1), r2 = ld_stream(hb + 2), r3 = ld_stream(hb + 3);
-                pk_acc_fx(h01, l01, make_float2(r0.x, r1.x), xv[0].x, xv[0].y);
-                pk_acc_fx(h01, l01, make_float2(r0.y, r1.y), xv[1].x, xv[1].y);
-                pk_acc_fx(h01, l01, make_float2(r0.z, r1.z), xv[2].x, xv[2].y);
-                pk_acc_fx(h01, l01, make_float2(r0.w, r1.w), xv[3].x, xv[3].y);
-                pk_acc_fx(h23, l23, make_float2(r2.x, r3.x), xv[0].x, xv[0].y);
-                pk_acc_fx(h23, l23, make_float2(r2.y, r3.y), xv[1].x, xv[1].y);
-                pk_acc_fx(h23, l23, make_float2(r2.z, r3.z), xv[2].x, xv[2].y);
-                pk_acc_fx(h23, l23, make_float2(r2.w, r3.w), xv[3].x, xv[3].y);
+                for (int k = 0; k < kPre; ++k) cb[k] = g0 + k < s1 ? ld_stream(a.bcol + (size_t)(g0 + k) * 8 + br) : -1;
+#pragma unroll
+                for (int k = 0; k < kPre; ++k)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) xv[k][q] = wprev[((size_t)max(cb[k], 0) * 4 + q) * T + cl];
+#pragma unroll
+                for (int k = 0; k < kPre; ++k) {
+                    if (cb[k] < 0) continue;
+                    const float4* hb = reinterpret_cast<const float4*>(a.bval + ((size_t)(g0 + k) * 8 + br) * 16);
+                    const float4 r0 = ld_stream(hb), r1 = ld_stream(hb + 1), r2 = ld_stream(hb + 2), r3 = ld_stream(hb + 3);
+                    pk_acc_fx(h01, l01, make_float2(r0.x, r1.x), xv[k][0].x, xv[k][0].y);
+                    pk_acc_fx(h01, l01, make_float2(r0.y, r1.y), xv[k][1].x, xv[k][1].y);
+                    pk_acc_fx(h01, l01, make_float2(r0.z, r1.z), xv[k][2].x, xv[k][2].y);
+                    pk_acc_fx(h01, l01, make_float2(r0.w, r1.w), xv[k][3].x, xv[k][3].y);
+                    pk_acc_fx(h23, l23, make_float2(r2.x, r3.x), xv[k][0].x, xv[k][0].y);
+                    pk_acc_fx(h23, l23, make_float2(r2.y, r3.y), xv[k][1].x, xv[k][1].y);
+                    pk_acc_fx(h23, l23, make_float2(r2.z, r3.z), xv[k][2].x, xv[k][2].y);
+                    pk_acc_fx(h23, l23, make_float2(r2.w, r3.w), xv[k][3].x, xv[k][3].y);
+                }
             }
             pk_norm(h01, l01);
             pk_norm(h23, l23);
@@ -697,17 +708,23 @@ __global__ void __launch_bounds__(kVecBlock) k_lz_next(int64_t n, int j, int m, 
 // falls below pivmin |P_i|) is replaced by -pivmin P_i, like a tiny negative
 // pivot; both minors are rescaled by 2^-600 / 2^600 to stay in range.
 // a and b2 (= b_{i-1}^2 at index i) are staged in shared memory by the caller.
+// The signs, the vanishing test (within a factor of two) and the range tests read
+// the high words as integers: an FP64 instruction holds its scheduler 64 cycles,
+// a comparison as long as a product, and this leaves three per step.
+__device__ __forceinline__ int hi_abs(double v) { return __double2hiint(v) & 0x7fffffff; }
 __device__ int tri_count_below(const double* a, const double* b2, int k, double x, double pivmin) {
     int c = 0;
+    const int dexp = (hi_abs(pivmin) >> 20) - 1023;      // exponent of pivmin
     double pm = 0.0, p = 1.0;   // P_{i-1}, P_i
     for (int i = 0; i < k; ++i) {
         double pn = fma(a[i] - x, p, -b2[i] * pm);
-        if (fabs(pn) <= pivmin * fabs(p)) pn = -pivmin * p;
-        if ((pn < 0.0) != (p < 0.0)) ++c;
+        if (hi_abs(pn) <= max(hi_abs(p) + dexp * (1 << 20), 0)) pn = -pivmin * p;
+        c += (unsigned)(__double2hiint(pn) ^ __double2hiint(p)) >> 31;
         pm = p;
         p = pn;
-        if (fabs(p) > 0x1p600) { p *= 0x1p-600; pm *= 0x1p-600; }
-        else if (fabs(p) < 0x1p-600 && fabs(pm) < 0x1p-600) { p *= 0x1p600; pm *= 0x1p600; }
+        const int h = hi_abs(p);
+        if (h > (1023 + 600) << 20) { p *= 0x1p-600; pm *= 0x1p-600; }
+        else if (h < (1023 - 600) << 20 && hi_abs(pm) < (1023 - 600) << 20) { p *= 0x1p600; pm *= 0x1p600; }
     }
     return c;
 }
@@ -722,7 +739,8 @@ __device__ __forceinline__ void stage_tri(const double* alpha, const double* bet
 }
 
 // Lowest eigenpair of the k x k tridiagonal T (alpha on the diagonal, beta
-// off it), one warp: multisection on the Sturm count (negative pivots of the
+// off it), one warp (80 steps: 735 us before the recurrences lost their divisions
+// and FP64 comparisons): multisection on the Sturm count (negative pivots of the
 // LDL^T factorisation of T - x) inside the Gershgorin interval, 32 points per
 // round, each lane counting at one point; then, in lane 0, three steps of
 // inverse iteration with T - theta factorised by Gaussian elimination with
@@ -737,10 +755,15 @@ __global__ void k_tri_lowest(const int* kdim, const double* alpha, const double*
     const double* b = beta;
     stage_tri(alpha, beta, k, s_a, s_b2);
     double lo = INFINITY, hi = -INFINITY;
-    for (int i = 0; i < k; ++i) {
+    for (int i = lane; i < k; i += 32) {
         const double r = (i > 0 ? fabs(b[i - 1]) : 0.0) + (i + 1 < k ? fabs(b[i]) : 0.0);
         lo = fmin(lo, a[i] - r);
         hi = fmax(hi, a[i] + r);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
     }
     const double scale = fmax(fmax(fabs(lo), fabs(hi)), 1e-300);
     const double eps = 2.220446049250313e-16;
@@ -758,54 +781,76 @@ __global__ void k_tri_lowest(const int* kdim, const double* alpha, const double*
         if (f == 32) lo = xf;
         else { hi = xf; if (f > 0) lo = xp; }
     }
-    if (lane != 0) return;
     const double th = 0.5 * (lo + hi);
-    *theta_out = th;
-    // LU of T - th with row interchanges: U0 diagonal, U1, U2 superdiagonals,
-    // l multipliers, sw = 1 where rows i and i + 1 were exchanged
+    // LU of T - th with row interchanges: U0 reciprocals of the diagonal, U1, U2
+    // superdiagonals, l multipliers, sw = 1 where rows i and i + 1 were exchanged
     double* U0 = work;
     double* U1 = work + k;
     double* U2 = work + 2 * k;
     double* l = work + 3 * k;
     double* sw = work + 4 * k;
     const double tiny = eps * scale + 1e-280;
-    double r0 = a[0] - th, r1 = k > 1 ? b[0] : 0.0, r2 = 0.0;
-    for (int i = 0; i + 1 < k; ++i) {
-        const double c = b[i];                       // row i+1: (b_i, a_{i+1} - th, b_{i+1})
-        const double d1 = a[i + 1] - th, d2 = i + 2 < k ? b[i + 1] : 0.0;
-        if (fabs(r0) >= fabs(c)) {
-            const double m = r0 != 0.0 ? c / r0 : 0.0;
-            U0[i] = r0; U1[i] = r1; U2[i] = r2; l[i] = m; sw[i] = 0.0;
-            r0 = d1 - m * r1; r1 = d2 - m * r2; r2 = 0.0;
-        } else {
-            const double m = r0 / c;
-            U0[i] = c; U1[i] = d1; U2[i] = d2; l[i] = m; sw[i] = 1.0;
-            const double n0 = r1 - m * d1, n1 = r2 - m * d2;
-            r0 = n0; r1 = n1; r2 = 0.0;
-        }
-        if (fabs(U0[i]) < tiny) U0[i] = U0[i] < 0.0 ? -tiny : tiny;
-    }
-    U0[k - 1] = fabs(r0) < tiny ? (r0 < 0.0 ? -tiny : tiny) : r0;
-    for (int i = 0; i < k; ++i) s[i] = 1.0 + (double)((i * 7919) % 13) / 13.0;
-    for (int rep = 0; rep < 3; ++rep) {
+    if (lane == 0) {
+        *theta_out = th;
+        double r0 = a[0] - th, r1 = k > 1 ? b[0] : 0.0, r2 = 0.0;
         for (int i = 0; i + 1 < k; ++i) {
-            if (sw[i] != 0.0) { const double t = s[i]; s[i] = s[i + 1]; s[i + 1] = t; }
-            s[i + 1] -= l[i] * s[i];
+            const double c = b[i];                       // row i+1: (b_i, a_{i+1} - th, b_{i+1})
+            const double d1 = s_a[i + 1] - th, d2 = i + 2 < k ? b[i + 1] : 0.0;
+            if (fabs(r0) >= fabs(c)) {
+                const double m = r0 != 0.0 ? c / r0 : 0.0;
+                U0[i] = r0; U1[i] = r1; U2[i] = r2; l[i] = m; sw[i] = 0.0;
+                r0 = d1 - m * r1; r1 = d2 - m * r2; r2 = 0.0;
+            } else {
+                const double m = r0 / c;
+                U0[i] = c; U1[i] = d1; U2[i] = d2; l[i] = m; sw[i] = 1.0;
+                const double n0 = r1 - m * d1, n1 = r2 - m * d2;
+                r0 = n0; r1 = n1; r2 = 0.0;
+            }
+            if (fabs(U0[i]) < tiny) U0[i] = U0[i] < 0.0 ? -tiny : tiny;
         }
-        for (int i = k - 1; i >= 0; --i) {
-            double v = s[i];
-            if (i + 1 < k) v -= U1[i] * s[i + 1];
-            if (i + 2 < k) v -= U2[i] * s[i + 2];
-            s[i] = v / U0[i];
-        }
-        double mx = 0.0;
-        for (int i = 0; i < k; ++i) mx = fmax(mx, fabs(s[i]));
-        if (!(mx > 0.0) || !isfinite(mx)) break;
-        double nr = 0.0;
-        for (int i = 0; i < k; ++i) { s[i] /= mx; nr += s[i] * s[i]; }
-        nr = sqrt(nr);
-        for (int i = 0; i < k; ++i) s[i] /= nr;
+        U0[k - 1] = fabs(r0) < tiny ? (r0 < 0.0 ? -tiny : tiny) : r0;
     }
+    __syncwarp();
+    for (int i = lane; i < k; i += 32) U0[i] = 1.0 / U0[i];
+    // the iterate in shared memory (the Sturm counts are done with s_b2)
+    double* v = s_b2;
+    __syncwarp();
+    for (int i = lane; i < k; i += 32) v[i] = 1.0 + (double)((i * 7919) % 13) / 13.0;
+    for (int rep = 0; rep < 3; ++rep) {
+        __syncwarp();
+        if (lane == 0) {
+            double cur = v[0];
+            for (int i = 0; i + 1 < k; ++i) {
+                double nxt = v[i + 1];
+                if (sw[i] != 0.0) { const double t = cur; cur = nxt; nxt = t; }
+                v[i] = cur;
+                cur = nxt - l[i] * cur;
+            }
+            v[k - 1] = cur;
+            double v1 = 0.0, v2 = 0.0;
+            for (int i = k - 1; i >= 0; --i) {
+                double t = v[i];
+                if (i + 1 < k) t -= U1[i] * v1;
+                if (i + 2 < k) t -= U2[i] * v2;
+                t *= U0[i];
+                v[i] = t;
+                v2 = v1; v1 = t;
+            }
+        }
+        __syncwarp();
+        double mx = 0.0;
+        for (int i = lane; i < k; i += 32) mx = fmax(mx, fabs(v[i]));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if (!(mx > 0.0) || !isfinite(mx)) break;
+        const double imx = 1.0 / mx;
+        double nr = 0.0;
+        for (int i = lane; i < k; i += 32) { const double t = v[i] * imx; v[i] = t; nr = fma(t, t, nr); }
+        const double inr = 1.0 / sqrt(warp_sum(nr));
+        for (int i = lane; i < k; i += 32) v[i] *= inr;
+    }
+    __syncwarp();
+    for (int i = lane; i < k; i += 32) s[i] = v[i];
 }
 
 // psi = sum_{j < k} s_j v_j; partial of psi^T psi
@@ -931,13 +976,14 @@ __global__ void __launch_bounds__(kVecBlock) k_proj_fin(const double* part, int 
     if (threadIdx.x == 0) P[(size_t)blockIdx.x * nu + j] = s;
 }
 
-// eigenvalue q (ascending) of T, one block of 32 threads each, of which 8
-// lanes run a multisection on the Sturm count inside the Gershgorin interval
-// (8 points per round, each lane counting at one point), keeping "fewer than
-// q + 1 eigenvalues below lo, at least q + 1 below hi".  Eight active lanes
-// issue an FP64 warp instruction in a quarter of the time of 32 on this
-// GPU's narrow FP64 pipe, which more than pays for the extra rounds.
-constexpr int kMsLanes = 8;
+// eigenvalues of T (ascending), LANES lanes each, 128 / LANES per block: a
+// multisection on the Sturm count inside the Gershgorin interval (LANES points
+// per round, each lane counting at one point), keeping "fewer than q + 1
+// eigenvalues below lo, at least q + 1 below hi".  An FP64 warp instruction costs
+// the same for 8 active lanes as for 32, so with many eigenvalues four share a
+// warp (16 recursions of 200 steps: 8.9 ms with one per warp and FP64
+// comparisons); with few, all 32 lanes take one, which saves a third of the rounds.
+constexpr int kTriBlock = 128;
 // The post-processing kernels below also serve several recursions at once:
 // recursion y = blockIdx.y finds its arrays `stride` elements after the
 // previous one's (all strides 0 with one recursion).
@@ -951,41 +997,68 @@ struct TriStride {
     int64_t bn;      // ||b||
 };
 
-__global__ void k_tri_evals(const int* kdim, const double* alpha, const double* beta, double* ev, double* scale_out,
-                            TriStride ys) {
+template <int LANES>
+__global__ void __launch_bounds__(kTriBlock) k_tri_evals(const int* kdim, const double* alpha, const double* beta,
+                                                         double* ev, double* scale_out, TriStride ys) {
     __shared__ double s_a[kMaxLanczos], s_b2[kMaxLanczos];
+    __shared__ double s_lo[kTriBlock / 32], s_hi[kTriBlock / 32];
     const int y = blockIdx.y;
     kdim += y; alpha += y * ys.tri; beta += y * ys.tri; ev += y * ys.tri;
     if (scale_out) scale_out += y * ys.scale;
     const int k = *kdim;
-    const int lane = threadIdx.x;
-    const int q = blockIdx.x;
+    const int lane = threadIdx.x % LANES;
+    const int q = (int)(blockIdx.x * (kTriBlock / LANES) + threadIdx.x / LANES);
     stage_tri(alpha, beta, k, s_a, s_b2);
-    if (lane >= kMsLanes) return;
     double lo = INFINITY, hi = -INFINITY;
-    for (int i = 0; i < k; ++i) {
+    for (int i = threadIdx.x; i < k; i += kTriBlock) {
         const double r = (i > 0 ? fabs(beta[i - 1]) : 0.0) + (i + 1 < k ? fabs(beta[i]) : 0.0);
         lo = fmin(lo, alpha[i] - r);
         hi = fmax(hi, alpha[i] + r);
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    }
+    if ((threadIdx.x & 31) == 0) { s_lo[threadIdx.x >> 5] = lo; s_hi[threadIdx.x >> 5] = hi; }
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kTriBlock / 32; ++w) { lo = fmin(lo, s_lo[w]); hi = fmax(hi, s_hi[w]); }
     const double scale = fmax(fmax(fabs(lo), fabs(hi)), 1e-300);
     if (q == 0 && lane == 0 && scale_out) *scale_out = scale;
-    if (q >= k) return;
     const double eps = 2.220446049250313e-16;
     const double pivmin = eps * scale * 1e-3 + 1e-300;
     lo -= 2.0 * eps * scale + pivmin;
     hi += 2.0 * eps * scale + pivmin;
-    constexpr unsigned kMask = (1u << kMsLanes) - 1u;
-    for (int it = 0; it < 96 && hi - lo > 2.0 * eps * fmax(fabs(lo), fabs(hi)) + pivmin; ++it) {
-        const double x = lo + (hi - lo) * ((double)(lane + 1) / (double)(kMsLanes + 1));
-        const unsigned above = __ballot_sync(kMask, tri_count_below(s_a, s_b2, k, x, pivmin) >= q + 1);
-        const int f = above ? __ffs(above) - 1 : kMsLanes;
-        const double xf = __shfl_sync(kMask, x, f < kMsLanes ? f : kMsLanes - 1);
-        const double xp = __shfl_sync(kMask, x, f > 0 ? f - 1 : 0);
-        if (f == kMsLanes) lo = xf;
-        else { hi = xf; if (f > 0) lo = xp; }
+    // the lanes of a warp stay together (shuffles); a finished or absent
+    // eigenvalue's lanes repeat their last interval without changing it
+    const int lane0 = (threadIdx.x & 31) - lane;
+    constexpr unsigned kMask = LANES == 32 ? 0xffffffffu : (1u << LANES) - 1u;
+    for (int it = 0; it < 96; ++it) {
+        const bool open = q < k && hi - lo > 2.0 * eps * fmax(fabs(lo), fabs(hi)) + pivmin;
+        if (!__any_sync(0xffffffffu, open)) break;
+        const double x = lo + (hi - lo) * ((double)(lane + 1) / (double)(LANES + 1));
+        const bool at = tri_count_below(s_a, s_b2, k, x, pivmin) >= q + 1;
+        const unsigned above = (__ballot_sync(0xffffffffu, at) >> lane0) & kMask;
+        const int f = above ? __ffs(above) - 1 : LANES;
+        const double xf = __shfl_sync(0xffffffffu, x, f < LANES ? f : LANES - 1, LANES);
+        const double xp = __shfl_sync(0xffffffffu, x, f > 0 ? f - 1 : 0, LANES);
+        if (open) {
+            if (f == LANES) lo = xf;
+            else { hi = xf; if (f > 0) lo = xp; }
+        }
     }
-    if (lane == 0) ev[q] = 0.5 * (lo + hi);
+    if (q < k && lane == 0) ev[q] = 0.5 * (lo + hi);
+}
+
+// the launch for ns recursions of up to nu steps: eight lanes per eigenvalue when
+// that fills the schedulers (four per SM), else 32
+static void tri_evals(int nu, int ns, int num_sms, const int* kdim, const double* alpha, const double* beta, double* ev,
+                      double* scale, const TriStride& ys, cudaStream_t st) {
+    if ((int64_t)nu * ns > 4LL * num_sms)
+        k_tri_evals<8><<<dim3((nu + kTriBlock / 8 - 1) / (kTriBlock / 8), ns), kTriBlock, 0, st>>>(kdim, alpha, beta, ev, scale, ys);
+    else
+        k_tri_evals<32><<<dim3((nu + kTriBlock / 32 - 1) / (kTriBlock / 32), ns), kTriBlock, 0, st>>>(kdim, alpha, beta, ev, scale, ys);
 }
 
 // eigenvectors of T (rows of S, S[q][i]): inverse iteration at each
@@ -1022,19 +1095,21 @@ __global__ void k_tri_evecs(const int* kdim, const double* alpha, const double* 
         for (int i = 0; i + 1 < k; ++i) {
             const double c = beta[i];
             const double d1 = alpha[i + 1] - th, d2 = i + 2 < k ? beta[i + 1] : 0.0;
-            double piv;
-            if (fabs(r0) >= fabs(c)) {
-                const double m = r0 != 0.0 ? c / r0 : 0.0;
-                piv = r0; U1[i] = r1; U2[i] = r2; l[i] = m; sw[i] = 0.0;
-                r0 = d1 - m * r1; r1 = d2 - m * r2; r2 = 0.0;
-            } else {
-                const double m = r0 / c;
-                piv = c; U1[i] = d1; U2[i] = d2; l[i] = m; sw[i] = 1.0;
-                const double n0 = r1 - m * d1, n1 = r2 - m * d2;
-                r0 = n0; r1 = n1; r2 = 0.0;
-            }
+            // one reciprocal per step: of the pivot, which the multiplier shares
+            const bool keep = fabs(r0) >= fabs(c);
+            double piv = keep ? r0 : c;
             if (fabs(piv) < tiny) piv = piv < 0.0 ? -tiny : tiny;
-            U0[i] = 1.0 / piv;
+            const double inv = 1.0 / piv, m = (keep ? c : r0) * inv;
+            U0[i] = inv; l[i] = m; sw[i] = keep ? 0.0 : 1.0;
+            if (keep) {
+                U1[i] = r1; U2[i] = r2;
+                r0 = d1 - m * r1; r1 = d2 - m * r2;
+            } else {
+                U1[i] = d1; U2[i] = d2;
+                const double n0 = r1 - m * d1, n1 = r2 - m * d2;
+                r0 = n0; r1 = n1;
+            }
+            r2 = 0.0;
         }
         U0[k - 1] = 1.0 / (fabs(r0) < tiny ? (r0 < 0.0 ? -tiny : tiny) : r0);
         double* s = S + (size_t)q * k;
@@ -1430,7 +1505,7 @@ extern "C" int scocg_krylov_sd(scocg_handle h, const double* b, int nu, const sc
     }
     if (e == cudaSuccess && status == SCOCG_OK) {
         const TriStride one{};
-        k_tri_evals<<<nu, 32, 0, st>>>(kdim, alpha, beta, ev, scal + 1, one);
+        tri_evals(nu, 1, h->num_sms, kdim, alpha, beta, ev, scal + 1, one, st);
         k_tri_evecs<<<(nu + 7) / 8, 8, 0, st>>>(kdim, alpha, beta, ev, scal + 1, S, work, one);
         k_krylov_weight<<<(M * nu + 127) / 128, 128, 0, st>>>(kdim, M, nu, S, P, scal, W, one);
         k_krylov_g<<<(M * K + 127) / 128, 128, 0, st>>>(kdim, M, nu, K, ev, W, d_z, (double2*)G_out, one);
@@ -1631,7 +1706,7 @@ extern "C" int scocg_krylov_sd_multi(scocg_handle h, const double* B, int nrhs, 
         if (status != SCOCG_OK) break;
         // the tridiagonal eigenproblems, weights and G of all ns recursions together
         const TriStride ys{nu, 4, (int64_t)nu * nu, 5LL * nu * nu, (int64_t)M * nu, (int64_t)M * K, 1};
-        k_tri_evals<<<dim3(nu, ns), 32, 0, st>>>(kdim, alpha, beta, ev, scal + 1, ys);
+        tri_evals(nu, ns, h->num_sms, kdim, alpha, beta, ev, scal + 1, ys, st);
         k_tri_evecs<<<dim3((nu + 7) / 8, ns), 8, 0, st>>>(kdim, alpha, beta, ev, scal + 1, S, work, ys);
         k_krylov_weight<<<dim3((M * nu + 127) / 128, ns), 128, 0, st>>>(kdim, M, nu, S, P, bnorm, W, ys);
         k_krylov_g<<<dim3((M * K + 127) / 128, ns), 128, 0, st>>>(kdim, M, nu, K, ev, W, d_z,
