@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(kVecBlock) k_csr_hx(int64_t n, const int* rowp
             acc = fma(xi, yi, acc);
         }
     }
-    block_partial(acc, part);
+    block_total(acc, part);
 }
 
 __device__ __forceinline__ bool lead() { return blockIdx.x == 0 && threadIdx.x == 0; }
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(kVecBlock) k_bsr4_hx(int64_t nunits, const int
             acc = fma(xi, yi, acc);
         }
     }
-    block_partial(acc, part);
+    block_total(acc, part);
 }
 
 // KR-SD's Lanczos recursion in one cooperative launch (4x4-blocked layout,
@@ -635,15 +635,15 @@ __global__ void k_to_slots(int64_t n, int T, int nslot, const double* x, double*
 __global__ void __launch_bounds__(kVecBlock) k_norm_part(int64_t n, const double* x, double* part) {
     double acc = 0.0;
     GRID_STRIDE(i, n) { const double v = x[i]; acc = fma(v, v, acc); }
-    block_partial(acc, part);
+    block_total(acc, part);
 }
 
 // dst = src / sqrt(sum of the partials); dst left as it is when that sum is
 // zero or not finite (*ok = 0, written by the lead thread)
 __global__ void __launch_bounds__(kVecBlock) k_scale_to(int64_t n, const double* src, double* dst,
-                                                        const double* part, int G, int* ok) {
+                                                        const double* part, int* ok) {
     __shared__ double s_inv;
-    const double s = sum_partials(part, G);
+    const double s = total_of(part);
     const bool good = s > 0.0 && isfinite(s);
     if (lead() && ok) *ok = good;
     if (!good) return;
@@ -653,12 +653,18 @@ __global__ void __launch_bounds__(kVecBlock) k_scale_to(int64_t n, const double*
     GRID_STRIDE(i, n) dst[i] = src[i] * inv;
 }
 
-// alpha_j = sum(part); w -= alpha_j v_j; partial of w^T w
-__global__ void __launch_bounds__(kVecBlock) k_lz_ortho(int64_t n, int j, const double* v, double* w,
-                                                        const double* part, int G, const int* stop, double* alpha,
-                                                        double* part2) {
-    if (stop[j]) return;
-    const double a = sum_partials(part, G);
+// alpha_j = sum(part); w -= alpha_j v_j; ||w||^2 and, in the block that completes
+// it, beta_j = ||w||.  The recursion ends after step j when j + 1 = m or
+// beta_j <= 1e-12 * max_i (|alpha_i| + beta_i + beta_{i-1}) (an invariant
+// subspace, or a non-finite value).
+__global__ void __launch_bounds__(kVecBlock) k_lz_ortho(int64_t n, int j, int m, const double* v, double* w,
+                                                        const double* part, int* stop, double* alpha, double* beta,
+                                                        double* tnorm, int* kdim, double* inv_beta, double* part2) {
+    if (stop[j]) {
+        if (lead()) stop[j + 1] = 1;
+        return;
+    }
+    const double a = total_of(part);
     if (lead()) alpha[j] = a;
     double acc = 0.0;
     GRID_STRIDE(i, n) {
@@ -666,38 +672,24 @@ __global__ void __launch_bounds__(kVecBlock) k_lz_ortho(int64_t n, int j, const 
         w[i] = wi;
         acc = fma(wi, wi, acc);
     }
-    block_partial(acc, part2);
+    const bool last = block_total(acc, part2);
+    if (last && threadIdx.x == 0) {   // one thread of the launch: roots and divisions are long FP64 chains
+        const double b = sqrt(total_of(part2));
+        const double tn = fmax(j ? tnorm[j - 1] : 0.0, fabs(a) + b + (j ? beta[j - 1] : 0.0));
+        const bool end = (j + 1 == m) || !(b > 1e-12 * tn);
+        beta[j] = b;
+        tnorm[j] = tn;
+        stop[j + 1] = end;
+        if (end) *kdim = j + 1;
+        *inv_beta = 1.0 / b;
+    }
 }
 
-// beta_j = sqrt(sum(part2)); the recursion ends after step j when j + 1 = m or
-// beta_j <= 1e-12 * max_i (|alpha_i| + beta_i + beta_{i-1}) (an invariant
-// subspace, or a non-finite value); else v_{j+1} = w / beta_j.
-__global__ void __launch_bounds__(kVecBlock) k_lz_next(int64_t n, int j, int m, const double* w, double* vnext,
-                                                       const double* part2, int G, const double* alpha, double* beta,
-                                                       double* tnorm, int* stop, int* kdim) {
-    if (stop[j]) {
-        if (lead()) stop[j + 1] = 1;
-        return;
-    }
-    __shared__ double s_inv;
-    __shared__ int s_end;
-    const double bsq = sum_partials(part2, G);
-    if (threadIdx.x == 0) {   // one thread: roots and divisions are long FP64 chains
-        const double b = sqrt(bsq);
-        const double tn = fmax(j ? tnorm[j - 1] : 0.0, fabs(alpha[j]) + b + (j ? beta[j - 1] : 0.0));
-        const bool end = (j + 1 == m) || !(b > 1e-12 * tn);
-        if (blockIdx.x == 0) {
-            beta[j] = b;
-            tnorm[j] = tn;
-            stop[j + 1] = end;
-            if (end) *kdim = j + 1;
-        }
-        s_end = end;
-        s_inv = 1.0 / b;
-    }
-    __syncthreads();
-    if (s_end) return;
-    const double inv = s_inv;
+// v_{j+1} = w / beta_j, unless the recursion ended with step j
+__global__ void __launch_bounds__(kVecBlock) k_lz_next(int64_t n, int j, const double* w, double* vnext,
+                                                       const int* stop, const double* inv_beta) {
+    if (stop[j + 1]) return;
+    const double inv = *inv_beta;
     GRID_STRIDE(i, n) vnext[i] = w[i] * inv;
 }
 
@@ -867,26 +859,26 @@ __global__ void __launch_bounds__(kVecBlock) k_ritz(int64_t n, const int* kdim, 
         psi[i] = v;
         acc = fma(v, v, acc);
     }
-    block_partial(acc, part);
+    block_total(acc, part);
 }
 
 // E = sum(part) (= psi^T H psi with h = H psi); partial of ||h - E psi||^2
 __global__ void __launch_bounds__(kVecBlock) k_resid(int64_t n, const double* psi, const double* h,
-                                                     const double* part, int G, double* part2, double* E_out) {
-    const double E = sum_partials(part, G);
+                                                     const double* part, double* part2, double* E_out) {
+    const double E = total_of(part);
     if (lead()) *E_out = E;
     double acc = 0.0;
     GRID_STRIDE(i, n) {
         const double r = fma(-E, psi[i], h[i]);
         acc = fma(r, r, acc);
     }
-    block_partial(acc, part2);
+    block_total(acc, part2);
 }
 
-// *out = sqrt(sum(part)) (one block) or the plain sum
-__global__ void __launch_bounds__(kVecBlock) k_sum_store(const double* part, int G, double* out, int take_sqrt) {
-    const double s = sum_partials(part, G);
-    if (threadIdx.x == 0) *out = take_sqrt ? sqrt(s) : s;
+// *out = sqrt(sum(part)) or the plain sum (one thread)
+__global__ void k_sum_store(const double* part, double* out, int take_sqrt) {
+    const double s = total_of(part);
+    *out = take_sqrt ? sqrt(s) : s;
 }
 
 // y = 0; r = p = psi; partial of r^T r
@@ -898,17 +890,17 @@ __global__ void __launch_bounds__(kVecBlock) k_cg_init(int64_t n, const double* 
         y[i] = 0.0; r[i] = v; p[i] = v;
         acc = fma(v, v, acc);
     }
-    block_partial(acc, part);
+    block_total(acc, part);
 }
 
 // step s: pq = p^T q (q = (H - sigma) p); breakdown when pq <= 0 or not finite;
 // else gamma = rr_s / pq, y += gamma p, r -= gamma q, partial of r^T r
 __global__ void __launch_bounds__(kVecBlock) k_cg_xr(int64_t n, int s, double* y, double* r, const double* p,
-                                                     const double* q, const double* part, int G, const double* rr,
+                                                     const double* q, const double* part, const double* rr,
                                                      const int* cgstop, int* cgbrk, double* part2) {
     if (cgstop[s]) return;
     __shared__ double s_g;
-    const double pq = sum_partials(part, G);
+    const double pq = total_of(part);
     const bool brk = !(pq > 0.0) || !isfinite(pq);
     if (lead()) cgbrk[s] = brk;
     if (brk) return;
@@ -922,19 +914,19 @@ __global__ void __launch_bounds__(kVecBlock) k_cg_xr(int64_t n, int s, double* y
         r[i] = ri;
         acc = fma(ri, ri, acc);
     }
-    block_partial(acc, part2);
+    block_total(acc, part2);
 }
 
 // rr_{s+1} = sum(part2); p = r + (rr_{s+1} / rr_s) p; the solve ends after
 // step s on a breakdown or when rr_{s+1} <= (1e-10)^2 rr_0
 __global__ void __launch_bounds__(kVecBlock) k_cg_p(int64_t n, int s, const double* r, double* p, const double* part2,
-                                                    int G, double* rr, int* cgstop, const int* cgbrk) {
+                                                    double* rr, int* cgstop, const int* cgbrk) {
     if (cgstop[s] || cgbrk[s]) {
         if (lead()) cgstop[s + 1] = 1;
         return;
     }
     __shared__ double s_be;
-    const double rn = sum_partials(part2, G);
+    const double rn = total_of(part2);
     if (threadIdx.x == 0) {   // one thread: divisions are long FP64 chains
         s_be = rn / rr[s];
         if (blockIdx.x == 0) {
@@ -1268,7 +1260,7 @@ extern "C" int scocg_ground_state(scocg_handle h, const double* v0, double* psi_
         }
         cv.take(sizeof(double) * (size_t)mm * n);
         for (int v = 0; v < 5; ++v) cv.take(sizeof(double) * n);
-        cv.take(sizeof(double) * (9 * (size_t)mm + 4 + 2 * (size_t)Gh + cg_steps + 1));
+        cv.take(sizeof(double) * (9 * (size_t)mm + 4 + 2 * (size_t)(Gh + kPartHead) + cg_steps + 1));
         cv.take(sizeof(int) * ((size_t)mm + 3 + 2 * (size_t)cg_steps + 1));
     }
     char* base = cv.base;
@@ -1281,9 +1273,9 @@ extern "C" int scocg_ground_state(scocg_handle h, const double* v0, double* psi_
     double* p = (double*)cv.take(sizeof(double) * n);
     GroundScalars S;
     {
-        double* d = (double*)cv.take(sizeof(double) * (9 * (size_t)mm + 4 + 2 * (size_t)Gh + cg_steps + 1));
+        double* d = (double*)cv.take(sizeof(double) * (9 * (size_t)mm + 4 + 2 * (size_t)(Gh + kPartHead) + cg_steps + 1));
         S.alpha = d; S.beta = d + mm; S.tnorm = d + 2 * mm; S.s = d + 3 * mm; S.work = d + 4 * mm;
-        S.scal = d + 9 * mm; S.part = S.scal + 4; S.part2 = S.part + Gh; S.rr = S.part2 + Gh;
+        S.scal = d + 9 * mm; S.part = S.scal + 4 + kPartHead; S.part2 = S.part + Gh + kPartHead; S.rr = S.part2 + Gh;
         int* q = (int*)cv.take(sizeof(int) * ((size_t)mm + 3 + 2 * (size_t)cg_steps + 1));
         S.stop = q; S.kdim = q + mm + 1; S.ok = S.kdim + 1; S.cgstop = S.ok + 1; S.cgbrk = S.cgstop + cg_steps + 1;
     }
@@ -1292,6 +1284,8 @@ extern "C" int scocg_ground_state(scocg_handle h, const double* v0, double* psi_
     cudaError_t e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
     if (e == cudaSuccess) e = cudaMemcpyAsync(psi, v0, sizeof(double) * n, cudaMemcpyDeviceToDevice, st);
+    for (double* pt : {S.part, S.part2})
+        if (e == cudaSuccess) e = cudaMemsetAsync(pt - kPartHead, 0, sizeof(double) * kPartHead, st);
     if (e == cudaSuccess) e = cudaEventRecord(e0, st);
     int status = SCOCG_NOT_CONVERGED;
     long long lanczos_total = 0, cg_total = 0;
@@ -1302,7 +1296,7 @@ extern "C" int scocg_ground_state(scocg_handle h, const double* v0, double* psi_
         ++cycles;
         // v_0 = psi / ||psi||
         k_norm_part<<<G, kVecBlock, 0, st>>>(n, psi, S.part);
-        k_scale_to<<<G, kVecBlock, 0, st>>>(n, psi, V, S.part, G, S.ok);
+        k_scale_to<<<G, kVecBlock, 0, st>>>(n, psi, V, S.part, S.ok);
         if (cyc == 0) {   // a zero or non-finite start vector is an invalid argument
             int ok = 0;
             e = cudaMemcpyAsync(&ok, S.ok, sizeof(int), cudaMemcpyDeviceToHost, st);
@@ -1317,19 +1311,20 @@ extern "C" int scocg_ground_state(scocg_handle h, const double* v0, double* psi_
             const double* vj = V + (size_t)j * n;
             e = hx(h, vj, w, j ? vj - n : nullptr, j ? S.beta + j - 1 : nullptr, 0.0, S.stop + j, S.part, Gh);
             if (e != cudaSuccess) break;
-            k_lz_ortho<<<G, kVecBlock, 0, st>>>(n, j, vj, w, S.part, Gh, S.stop, S.alpha, S.part2);
-            k_lz_next<<<G, kVecBlock, 0, st>>>(n, j, mm, w, j + 1 < mm ? V + (size_t)(j + 1) * n : w, S.part2, G,
-                                               S.alpha, S.beta, S.tnorm, S.stop, S.kdim);
+            k_lz_ortho<<<G, kVecBlock, 0, st>>>(n, j, mm, vj, w, S.part, S.stop, S.alpha, S.beta, S.tnorm, S.kdim,
+                                                S.scal + 3, S.part2);
+            if (j + 1 < mm)
+                k_lz_next<<<G, kVecBlock, 0, st>>>(n, j, w, V + (size_t)(j + 1) * n, S.stop, S.scal + 3);
             e = cudaGetLastError();
         }
         if (e != cudaSuccess) break;
         k_tri_lowest<<<1, 32, 0, st>>>(S.kdim, S.alpha, S.beta, S.s, S.work, S.scal);
         k_ritz<<<G, kVecBlock, 0, st>>>(n, S.kdim, S.s, V, w, S.part);
-        k_scale_to<<<G, kVecBlock, 0, st>>>(n, w, psi, S.part, G, S.ok);
+        k_scale_to<<<G, kVecBlock, 0, st>>>(n, w, psi, S.part, S.ok);
         e = hx(h, psi, w, nullptr, nullptr, 0.0, nullptr, S.part, Gh);
         if (e != cudaSuccess) break;
-        k_resid<<<G, kVecBlock, 0, st>>>(n, psi, w, S.part, Gh, S.part2, S.scal + 1);
-        k_sum_store<<<1, kVecBlock, 0, st>>>(S.part2, G, S.scal + 2, 1);
+        k_resid<<<G, kVecBlock, 0, st>>>(n, psi, w, S.part, S.part2, S.scal + 1);
+        k_sum_store<<<1, 1, 0, st>>>(S.part2, S.scal + 2, 1);
         double sc[3];
         int kd = 0;
         e = cudaGetLastError();
@@ -1346,18 +1341,18 @@ extern "C" int scocg_ground_state(scocg_handle h, const double* v0, double* psi_
         // inverse iteration: CG on (H - sigma) y = psi
         const double sigma = E - res;
         k_cg_init<<<G, kVecBlock, 0, st>>>(n, psi, y, r, p, S.part);
-        k_sum_store<<<1, kVecBlock, 0, st>>>(S.part, G, S.rr, 0);
+        k_sum_store<<<1, 1, 0, st>>>(S.part, S.rr, 0);
         e = cudaMemsetAsync(S.cgstop, 0, sizeof(int) * (2 * (size_t)cg_steps + 1), st);
         for (int s = 0; s < cg_steps && e == cudaSuccess; ++s) {
             e = hx(h, p, w, nullptr, nullptr, sigma, S.cgstop + s, S.part, Gh);
             if (e != cudaSuccess) break;
-            k_cg_xr<<<G, kVecBlock, 0, st>>>(n, s, y, r, p, w, S.part, Gh, S.rr, S.cgstop, S.cgbrk, S.part2);
-            k_cg_p<<<G, kVecBlock, 0, st>>>(n, s, r, p, S.part2, G, S.rr, S.cgstop, S.cgbrk);
+            k_cg_xr<<<G, kVecBlock, 0, st>>>(n, s, y, r, p, w, S.part, S.rr, S.cgstop, S.cgbrk, S.part2);
+            k_cg_p<<<G, kVecBlock, 0, st>>>(n, s, r, p, S.part2, S.rr, S.cgstop, S.cgbrk);
             e = cudaGetLastError();
         }
         if (e != cudaSuccess) break;
         k_norm_part<<<G, kVecBlock, 0, st>>>(n, y, S.part);
-        k_scale_to<<<G, kVecBlock, 0, st>>>(n, y, psi, S.part, G, S.ok);   // psi kept if y = 0
+        k_scale_to<<<G, kVecBlock, 0, st>>>(n, y, psi, S.part, S.ok);   // psi kept if y = 0
         e = cudaMemcpyAsync(host_stop.data(), S.cgstop, sizeof(int) * (cg_steps + 1), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e == cudaSuccess) {
@@ -1441,8 +1436,8 @@ extern "C" int scocg_krylov_sd(scocg_handle h, const double* b, int nu, const sc
         tnorm = (double*)cv.take(sizeof(double) * nu);
         ev = (double*)cv.take(sizeof(double) * nu);
         scal = (double*)cv.take(sizeof(double) * 4);
-        part = (double*)cv.take(sizeof(double) * Gh);
-        part2 = (double*)cv.take(sizeof(double) * Gh);
+        part = (double*)cv.take(sizeof(double) * (Gh + kPartHead)) + kPartHead;
+        part2 = (double*)cv.take(sizeof(double) * (Gh + kPartHead)) + kPartHead;
         partM = (double*)cv.take(sizeof(double) * (size_t)M * G);
         stop = (int*)cv.take(sizeof(int) * (nu + 1));
         kdim = (int*)cv.take(sizeof(int));
@@ -1459,13 +1454,15 @@ extern "C" int scocg_krylov_sd(scocg_handle h, const double* b, int nu, const sc
         e = cudaMemcpyAsync(d_idx, proj_idx, sizeof(int64_t) * M, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(stop, 0, sizeof(int) * (nu + 1), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(P, 0, sizeof(double) * (size_t)M * nu, st);
+    for (double* pt : {part, part2})
+        if (e == cudaSuccess) e = cudaMemsetAsync(pt - kPartHead, 0, sizeof(double) * kPartHead, st);
     if (e == cudaSuccess) e = cudaEventRecord(e0, st);
     int status = SCOCG_OK;
     if (e == cudaSuccess) {
         // v_0 = b / ||b||, ||b|| kept for the weights
         k_norm_part<<<G, kVecBlock, 0, st>>>(n, b, part);
-        k_sum_store<<<1, kVecBlock, 0, st>>>(part, G, scal, 1);
-        k_scale_to<<<G, kVecBlock, 0, st>>>(n, b, vb[0], part, G, kdim);
+        k_sum_store<<<1, 1, 0, st>>>(part, scal, 1);
+        k_scale_to<<<G, kVecBlock, 0, st>>>(n, b, vb[0], part, kdim);
         int ok = 0;
         e = cudaMemcpyAsync(&ok, kdim, sizeof(int), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -1499,8 +1496,8 @@ extern "C" int scocg_krylov_sd(scocg_handle h, const double* b, int nu, const sc
         }
         e = hx(h, vj, w, j ? vb[(j + 2) % 3] : nullptr, j ? beta + j - 1 : nullptr, 0.0, stop + j, part, Gh);
         if (e != cudaSuccess) break;
-        k_lz_ortho<<<G, kVecBlock, 0, st>>>(n, j, vj, w, part, Gh, stop, alpha, part2);
-        k_lz_next<<<G, kVecBlock, 0, st>>>(n, j, nu, w, vb[(j + 1) % 3], part2, G, alpha, beta, tnorm, stop, kdim);
+        k_lz_ortho<<<G, kVecBlock, 0, st>>>(n, j, nu, vj, w, part, stop, alpha, beta, tnorm, kdim, scal + 3, part2);
+        if (j + 1 < nu) k_lz_next<<<G, kVecBlock, 0, st>>>(n, j, w, vb[(j + 1) % 3], stop, scal + 3);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && status == SCOCG_OK) {

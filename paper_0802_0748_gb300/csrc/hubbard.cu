@@ -130,8 +130,8 @@ struct ApplyHubbard {
 
     __device__ __forceinline__ bool operator()(int64_t unit, int lane, float4 zs, const float4* x, int64_t& row,
                                                float4& w) const {
-        const int u = (int)(unit % D_up);
-        const int d = (int)(unit / D_up) * 32 + lane;
+        const int u = (int)((uint32_t)unit % (uint32_t)D_up);
+        const int d = (int)((uint32_t)unit / (uint32_t)D_up) * 32 + lane;
         if (d >= D_dn) return false;
         row = (int64_t)u * D_dn + d;
         const uint32_t su = st_up[u], sd = st_dn[d];
@@ -164,19 +164,19 @@ struct ApplyHubbard {
     // the row whose term (unit, lane) adds to the r^T q partial of phase A
     // (the tile-major order of the one-pass apply and of pass 2)
     __device__ __forceinline__ bool row_of(int64_t unit, int lane, int64_t& row) const {
-        const int u = (int)(unit % D_up), d = (int)(unit / D_up) * 32 + lane;
+        const int u = (int)((uint32_t)unit % (uint32_t)D_up), d = (int)((uint32_t)unit / (uint32_t)D_up) * 32 + lane;
         row = (int64_t)u * D_dn + d;
         return d < D_dn;
     }
     __device__ __forceinline__ bool rc_rows(int64_t unit, int lane, int& u, int& d) const {
         const int tiles = (D_dn + 31) / 32;
-        u = (int)(unit / tiles);
-        d = (int)(unit % tiles) * 32 + lane;
+        u = (int)((uint32_t)unit / (uint32_t)tiles);
+        d = (int)((uint32_t)unit % (uint32_t)tiles) * 32 + lane;
         return d < D_dn;
     }
     __device__ __forceinline__ bool rc_tiles(int64_t unit, int lane, int& u, int& d) const {
-        u = (int)(unit % D_up);
-        d = (int)(unit / D_up) * 32 + lane;
+        u = (int)((uint32_t)unit % (uint32_t)D_up);
+        d = (int)((uint32_t)unit / (uint32_t)D_up) * 32 + lane;
         return d < D_dn;
     }
     __device__ __forceinline__ int diag_index(int u, int d) const {
@@ -272,8 +272,8 @@ struct ApplyHubbard {
     __device__ __forceinline__ bool operator()(int64_t unit, int lane, VV zs, const VV* x, int64_t& row,
                                                VV& w) const {
         using T = typename Scal<VV>::T;
-        const int u = (int)(unit % D_up);
-        const int d = (int)(unit / D_up) * 32 + lane;
+        const int u = (int)((uint32_t)unit % (uint32_t)D_up);
+        const int d = (int)((uint32_t)unit / (uint32_t)D_up) * 32 + lane;
         if (d >= D_dn) return false;
         row = (int64_t)u * D_dn + d;
         const uint32_t su = st_up[u], sd = st_dn[d];
@@ -439,8 +439,8 @@ __global__ void __launch_bounds__(kVecBlock) k_hub_hx(ApplyHubbard<double> ap, i
     const double bp = (xprev && beta) ? *beta : 0.0;
     double acc = 0.0;
     for (int64_t unit = w0; unit < nunits; unit += nw) {
-        const int u = (int)(unit % ap.D_up);
-        const int d = (int)(unit / ap.D_up) * 32 + lane;
+        const int u = (int)((uint32_t)unit % (uint32_t)ap.D_up);
+        const int d = (int)((uint32_t)unit / (uint32_t)ap.D_up) * 32 + lane;
         if (d >= ap.D_dn) continue;
         const int64_t row = (int64_t)u * ap.D_dn + d;
         const uint32_t su = ap.st_up[u], sd = ap.st_dn[d];
@@ -460,7 +460,7 @@ __global__ void __launch_bounds__(kVecBlock) k_hub_hx(ApplyHubbard<double> ap, i
         y[row] = yi;
         acc = fma(xi, yi, acc);
     }
-    block_partial(acc, part);
+    block_total(acc, part);
 }
 
 cudaError_t hubbard_hx(const Hubbard& hb, const double* x, double* y, const double* xprev, const double* beta,

@@ -140,11 +140,11 @@ struct ApplyHubbard2 {
     __device__ __forceinline__ void unit_rc(int64_t unit, int lane, int& u, int& d) const {
 #if SCOCG_H2_UMAJOR
         const int tiles = (D_dn + 31) / 32;
-        u = (int)(unit / tiles);
-        d = (int)(unit % tiles) * 32 + lane;
+        u = (int)((uint32_t)unit / (uint32_t)tiles);
+        d = (int)((uint32_t)unit % (uint32_t)tiles) * 32 + lane;
 #else
-        u = (int)(unit % D_up);
-        d = (int)(unit / D_up) * 32 + lane;
+        u = (int)((uint32_t)unit % (uint32_t)D_up);
+        d = (int)((uint32_t)unit / (uint32_t)D_up) * 32 + lane;
 #endif
     }
 
@@ -262,19 +262,19 @@ struct ApplyHubbard2 {
     // the row whose term (unit, lane) adds to the r^T q partial of phase A
     // (the tile-major order of the one-pass apply and of pass 2)
     __device__ __forceinline__ bool row_of(int64_t unit, int lane, int64_t& row) const {
-        const int u = (int)(unit % D_up), d = (int)(unit / D_up) * 32 + lane;
+        const int u = (int)((uint32_t)unit % (uint32_t)D_up), d = (int)((uint32_t)unit / (uint32_t)D_up) * 32 + lane;
         row = (int64_t)u * D_dn + d;
         return d < D_dn;
     }
     __device__ __forceinline__ bool rc_rows(int64_t unit, int lane, int& u, int& d) const {
         const int tiles = (D_dn + 31) / 32;
-        u = (int)(unit / tiles);
-        d = (int)(unit % tiles) * 32 + lane;
+        u = (int)((uint32_t)unit / (uint32_t)tiles);
+        d = (int)((uint32_t)unit % (uint32_t)tiles) * 32 + lane;
         return d < D_dn;
     }
     __device__ __forceinline__ bool rc_tiles(int64_t unit, int lane, int& u, int& d) const {
-        u = (int)(unit % D_up);
-        d = (int)(unit / D_up) * 32 + lane;
+        u = (int)((uint32_t)unit % (uint32_t)D_up);
+        d = (int)((uint32_t)unit / (uint32_t)D_up) * 32 + lane;
         return d < D_dn;
     }
     __device__ __forceinline__ float4 pass1_w(int u, int d, float4 zs, const float4* x) const {
@@ -567,7 +567,7 @@ __global__ void __launch_bounds__(kVecBlock, 4) k_hub2_hx2(ApplyHubbard2<double>
         y[row] = yi;
         acc = fma(x[row], yi, acc);
     }
-    block_partial(acc, part);
+    block_total(acc, part);
 }
 
 cudaError_t hubbard2_hx(const Hubbard& hb, const double* x, double* y, const double* xprev, const double* beta,
