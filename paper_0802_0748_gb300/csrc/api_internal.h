@@ -79,6 +79,7 @@ struct Hubbard {
     double* d_self2 = nullptr;         // [2][Dmax]: the diagonal terms of one spin alone
     float2* d_self2f = nullptr;        // [2][Dmax]: the same as float pairs (hi, lo)
     double* d_amp2 = nullptr;          // [nb][2][2] hoppings t_ab of each bond
+    int amp2_fp32 = 0;                 // every hopping is an FP32 value
     float2* d_amp2f = nullptr;         // [nb][2][2][2] the same with each sign, as (hi, hi, lo, lo) float4s
     double* d_cross2 = nullptr;        // [3][kCross2]: U c, U' c, V c for small integer counts c
     float2* d_cross2f = nullptr;       // the same as float pairs

@@ -25,9 +25,6 @@
 #include "vector_ops.cuh"
 #include "hubbard_basis.cuh"
 
-#ifndef SCOCG_RING_TWO_PASS
-#define SCOCG_RING_TWO_PASS 0
-#endif
 #ifndef SCOCG_HOP_GROUP
 #define SCOCG_HOP_GROUP 4
 #endif
@@ -153,121 +150,14 @@ struct ApplyHubbard {
         return true;
     }
 
-    // ---- two-pass form (phase A runs pass 1 over all units, a grid barrier,
-    // then pass 2; off for the ring, where one pass measured faster: 622 vs
-    // 686 us per iteration at 14 sites, while the two-orbital model gains).  Pass 1 visits units row-major
-    // (unit = u * tiles + tile: the CTAs share the rows x[u][:] of the down
-    // hops) and stores q = (z_s - diag) x + t (down-hop sum) + beta q_old;
-    // pass 2 visits them tile-major (unit = tile * D_up + u: the CTAs share the
-    // column tiles x[:][tile] of the up hops) and adds t (up-hop sum).
-    static constexpr bool kTwoPass = SCOCG_RING_TWO_PASS;
+    // one pass per apply (the two-pass form of the two-orbital model measured
+    // slower here: 686 against 622 us per iteration at 14 sites)
     // the row whose term (unit, lane) adds to the r^T q partial of phase A
-    // (the tile-major order of the one-pass apply and of pass 2)
     __device__ __forceinline__ bool row_of(int64_t unit, int lane, int64_t& row) const {
         const int u = (int)((uint32_t)unit % (uint32_t)D_up), d = (int)((uint32_t)unit / (uint32_t)D_up) * 32 + lane;
         row = (int64_t)u * D_dn + d;
         return d < D_dn;
     }
-    __device__ __forceinline__ bool rc_rows(int64_t unit, int lane, int& u, int& d) const {
-        const int tiles = (D_dn + 31) / 32;
-        u = (int)((uint32_t)unit / (uint32_t)tiles);
-        d = (int)((uint32_t)unit % (uint32_t)tiles) * 32 + lane;
-        return d < D_dn;
-    }
-    __device__ __forceinline__ bool rc_tiles(int64_t unit, int lane, int& u, int& d) const {
-        u = (int)((uint32_t)unit % (uint32_t)D_up);
-        d = (int)((uint32_t)unit / (uint32_t)D_up) * 32 + lane;
-        return d < D_dn;
-    }
-    __device__ __forceinline__ int diag_index(int u, int d) const {
-        const uint32_t su = st_up[u], sd = st_dn[d];
-        const uint32_t pu = partner(su), pd = partner(sd);
-        const int cu = __popc(su & sd);
-        const int cv = __popc(su & pu) + __popc(sd & pd) + __popc(su & pd) + __popc(sd & pu);
-        return cu * (4 * L + 1) + cv;
-    }
-    __device__ __forceinline__ double diag_of(int u, int d) const {
-        const uint32_t su = st_up[u], sd = st_dn[d];
-        const uint32_t pu = partner(su), pd = partner(sd);
-        const int cu = __popc(su & sd);
-        const int cv = __popc(su & pu) + __popc(sd & pd) + __popc(su & pd) + __popc(sd & pu);
-        return U * (double)cu + V * (double)cv;
-    }
-
-    __device__ __forceinline__ void pass1(int64_t unit, int lane, float4 zs, float4 bp, const float4* x,
-                                          float4* q) const {
-        int u, d;
-        if (!rc_rows(unit, lane, u, d)) return;
-        const int64_t row = (int64_t)u * D_dn + d;
-        float2 h = make_float2(0.f, 0.f), l = make_float2(0.f, 0.f);
-        hop_acc_df(hop_dn + (size_t)d * S, S, x + (size_t)u * D_dn, 1, D_dn, dbg, h, l);
-        pk_norm(h, l);
-        const float2 dg = diagf[diag_index(u, d)];
-        const dfs zr = df_add(cre(zs), dfs{-dg.x, -dg.y});
-        const float4 acc = vcfma(cpack(zr, cim(zs)), x[row], vzero<float4>());
-        float2 ah = hi2(acc), al = lo2(acc);
-        pk_acc_prod(ah, al, make_float2(t_hi, t_hi), make_float2(t_lo, t_lo), h, l);
-        pk_norm(ah, al);
-        q[row] = vcfma(bp, q[row], pk4(ah, al));
-    }
-    __device__ __forceinline__ bool pass2(int64_t unit, int lane, const float4* x, float4* q, int64_t& row,
-                                          float4& qn) const {
-        int u, d;
-        if (!rc_tiles(unit, lane, u, d)) return false;
-        row = (int64_t)u * D_dn + d;
-        float2 h = make_float2(0.f, 0.f), l = make_float2(0.f, 0.f);
-        hop_acc_df(hop_up + (size_t)u * S, S, x + d, D_dn, D_up, dbg, h, l);
-        pk_norm(h, l);
-        const float4 q1 = q[row];
-        float2 ah = hi2(q1), al = lo2(q1);
-        pk_acc_prod(ah, al, make_float2(t_hi, t_hi), make_float2(t_lo, t_lo), h, l);
-        pk_norm(ah, al);
-        qn = pk4(ah, al);
-        q[row] = qn;
-        return true;
-    }
-    // FP64 and complex64 vectors
-    template <typename VV>
-    __device__ __forceinline__ VV hop_sum_v(const int32_t* tab, const VV* base, int64_t stride, int64_t lim) const {
-        using T = typename Scal<VV>::T;
-        VV acc;
-        acc.x = 0; acc.y = 0;
-        for (int j = 0; j < S; ++j) {
-            const int e = tab[j];
-            if (e < 0) break;
-            if (!chk(dbg, 20, e >> 1, lim)) continue;
-            const VV xv = base[(int64_t)(e >> 1) * stride];
-            const T c = (e & 1) ? -(T)t : (T)t;
-            acc.x += c * xv.x; acc.y += c * xv.y;
-        }
-        return acc;
-    }
-    template <typename VV>
-    __device__ __forceinline__ void pass1(int64_t unit, int lane, VV zs, VV bp, const VV* x, VV* q) const {
-        using T = typename Scal<VV>::T;
-        int u, d;
-        if (!rc_rows(unit, lane, u, d)) return;
-        const int64_t row = (int64_t)u * D_dn + d;
-        const VV hs = hop_sum_v(hop_dn + (size_t)d * S, x + (size_t)u * D_dn, 1, D_dn);
-        const T zr = zs.x - (T)diag_of(u, d);
-        const VV xr = x[row];
-        VV w;
-        w.x = zr * xr.x - zs.y * xr.y + hs.x;
-        w.y = zr * xr.y + zs.y * xr.x + hs.y;
-        q[row] = vcfma(bp, q[row], w);
-    }
-    template <typename VV>
-    __device__ __forceinline__ bool pass2(int64_t unit, int lane, const VV* x, VV* q, int64_t& row, VV& qn) const {
-        int u, d;
-        if (!rc_tiles(unit, lane, u, d)) return false;
-        row = (int64_t)u * D_dn + d;
-        const VV hs = hop_sum_v(hop_up + (size_t)u * S, x + d, D_dn, D_up);
-        qn = q[row];
-        qn.x += hs.x; qn.y += hs.y;
-        q[row] = qn;
-        return true;
-    }
-
     template <typename VV>
     __device__ __forceinline__ bool operator()(int64_t unit, int lane, VV zs, const VV* x, int64_t& row,
                                                VV& w) const {

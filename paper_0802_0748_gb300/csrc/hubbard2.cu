@@ -41,9 +41,9 @@ constexpr int kMaxSites2 = 16;       // 2 ns <= 32 modes per spin
 constexpr int kMaxBonds2 = 32;       // amplitude index b*4 + a*2 + a' < 128 (7 bits)
 constexpr int kCross2 = 257;         // counts 0..256 of the cross-spin diagonal tables (8 per bond at most)
 #ifndef SCOCG_H2_GROUP
-#define SCOCG_H2_GROUP 4
+#define SCOCG_H2_GROUP 2   // hop entries of two rows read (and gathered) together
 #endif
-constexpr int kHop2Group = SCOCG_H2_GROUP;   // hop entries read (and gathered) together
+constexpr int kHop2Group = 4;   // the same of one row
 #ifndef SCOCG_H2_UMAJOR
 #define SCOCG_H2_UMAJOR 0
 #endif
@@ -130,6 +130,7 @@ struct ApplyHubbard2 {
     int S2, ns, D_up, D_dn;
     double J, Jp;
     float Jh, Jl, Ph, Pl;      // -J and -J' as float pairs (hi, lo)
+    int amp_fp32;              // every amplitude is an FP32 value (its low part is zero)
     int64_t n;
     unsigned long long* dbg;
 
@@ -155,8 +156,13 @@ struct ApplyHubbard2 {
         cp = __popc(su & (sd >> 1) & ev) + __popc(sd & (su >> 1) & ev);
         const uint32_t nu = nib_up[2 * (size_t)u], and_ = nib_dn[2 * (size_t)d + 1];
         int c = 0;
+        if (ns <= 8) {   // eight sites' nibbles as two packed byte products
+            constexpr uint32_t kNib = 0x0f0f0f0fu;
+            c = (int)__dp4a(nu & kNib, and_ & kNib, __dp4a((nu >> 4) & kNib, (and_ >> 4) & kNib, 0u));
+        } else {
 #pragma unroll 4
-        for (int i = 0; i < ns; ++i) c += (int)(((nu >> (4 * i)) & 15u) * ((and_ >> (4 * i)) & 15u));
+            for (int i = 0; i < ns; ++i) c += (int)(((nu >> (4 * i)) & 15u) * ((and_ >> (4 * i)) & 15u));
+        }
         cv = c;
     }
 
@@ -190,22 +196,37 @@ struct ApplyHubbard2 {
         }
     }
 
-    // joint moves (spin flip: J, pair hopping: J'), summed separately
+    // joint moves (spin flip: J, pair hopping: J'), summed separately; four sites'
+    // moves, then their gathers, are in flight together
     __device__ __forceinline__ void joint_df(int u, int d, const float4* x, float2& hj, float2& lj, float2& hp,
                                              float2& lp) const {
-        for (int i = 0; i < ns; ++i) {
-            const int32_t mu = orb_up[(size_t)i * D_up + u], md = orb_dn[(size_t)i * D_dn + d];
-            if (mu < 0 || md < 0) continue;
-            const int tu = mu >> 1, td = md >> 1;
-            if (!chk(dbg, 23, tu, D_up) || !chk(dbg, 24, td, D_dn)) continue;
-            const float4 xv = x[(size_t)tu * D_dn + td];
-            float2 t, er;
-            if ((mu & 1) != (md & 1)) {
-                pk_two_sum(hj, hi2(xv), t, er);
-                hj = t; lj = pk_add(lj, pk_add(er, lo2(xv)));
-            } else {
-                pk_two_sum(hp, hi2(xv), t, er);
-                hp = t; lp = pk_add(lp, pk_add(er, lo2(xv)));
+#ifndef SCOCG_H2_JOINT
+#define SCOCG_H2_JOINT 2
+#endif
+        constexpr int kG = SCOCG_H2_JOINT;
+        for (int i0 = 0; i0 < ns; i0 += kG) {
+            int32_t mu[kG], md[kG];
+            float4 xv[kG];
+#pragma unroll
+            for (int q = 0; q < kG; ++q) {
+                mu[q] = i0 + q < ns ? orb_up[(size_t)(i0 + q) * D_up + u] : -1;   // the same for the whole warp
+                md[q] = mu[q] >= 0 ? orb_dn[(size_t)(i0 + q) * D_dn + d] : -1;
+                if (md[q] >= 0 && (!chk(dbg, 23, mu[q] >> 1, D_up) || !chk(dbg, 24, md[q] >> 1, D_dn))) md[q] = -1;
+            }
+#pragma unroll
+            for (int q = 0; q < kG; ++q)
+                if (md[q] >= 0) xv[q] = x[(size_t)(mu[q] >> 1) * D_dn + (md[q] >> 1)];
+#pragma unroll
+            for (int q = 0; q < kG; ++q) {
+                if (md[q] < 0) continue;
+                float2 t, er;
+                if ((mu[q] & 1) != (md[q] & 1)) {
+                    pk_two_sum(hj, hi2(xv[q]), t, er);
+                    hj = t; lj = pk_add(lj, pk_add(er, lo2(xv[q])));
+                } else {
+                    pk_two_sum(hp, hi2(xv[q]), t, er);
+                    hp = t; lp = pk_add(lp, pk_add(er, lo2(xv[q])));
+                }
             }
         }
         pk_norm(hj, lj);
@@ -253,12 +274,125 @@ struct ApplyHubbard2 {
         return true;
     }
 
-    // ---- two-pass form used by the persistent solve: pass 1 over the units
-    // row-major (the CTAs share the rows x[u][:] of the down hops and the few
-    // rows of the joint moves) stores q = (z_s - diag) x - (down hops and
-    // joint moves) + beta q_old; pass 2 tile-major (the CTAs share the column
-    // tiles x[:][tile] of the up hops) subtracts the up hops.
+    // ---- two-pass form used by the persistent solve, kRows rows per lane and
+    // unit.  Pass 1 visits pairs of rows (u, u + 1) of a tile of 32 down ranks,
+    // row-major (the CTAs share the rows x[u][:] of the down hops and the few rows
+    // of the joint moves): a lane's down-hop list and its amplitudes are read once
+    // for both rows.  It stores q = (z_s - diag) x - (down hops and joint moves) +
+    // beta q_old.  Pass 2 visits pairs of tiles of one row u, tile-major (the CTAs
+    // share the column tiles x[:][tile] of the up hops): the up-hop list serves 64
+    // down ranks; it subtracts the up hops.  (One row per lane spent as much on the
+    // lists as on the arithmetic: 3 up / 4 down of the 8-site cluster 165 us per
+    // iteration.)
     static constexpr bool kTwoPass = true;
+    static constexpr int kRows = 2;
+    __device__ __forceinline__ int64_t units1() const { return (int64_t)((D_up + 1) / 2) * ((D_dn + 31) / 32); }
+    __device__ __forceinline__ int64_t units2() const { return (int64_t)D_up * ((D_dn + 63) / 64); }
+    // rank pair of pass 1's and pass 2's units: row k is (u + k, d) or (u, d + 32 k)
+    __device__ __forceinline__ void rc1(int64_t unit, int lane, int& u, int& d) const {
+        const uint32_t tiles = (uint32_t)(D_dn + 31) / 32;
+        u = 2 * (int)((uint32_t)unit / tiles);
+        d = (int)((uint32_t)unit % tiles) * 32 + lane;
+    }
+    __device__ __forceinline__ void rc2(int64_t unit, int lane, int& u, int& d) const {
+        u = (int)((uint32_t)unit % (uint32_t)D_up);
+        d = (int)((uint32_t)unit / (uint32_t)D_up) * 64 + lane;
+    }
+    __device__ __forceinline__ bool row2_of(int64_t unit, int lane, int k, int64_t& row) const {
+        int u, d;
+        rc2(unit, lane, u, d);
+        row = (int64_t)u * D_dn + d + 32 * k;
+        return d + 32 * k < D_dn;
+    }
+    // Hop sums of two rows at base and base + off (off = 0: one row, its sum
+    // twice).  An ended list reads entry 0 and adds zero times it: no branch per
+    // entry, whose divergence took a fifth of the issue slots.
+    __device__ __forceinline__ void hops2_df(const int32_t* tab, int64_t tstride, const float4* base, int64_t off,
+                                             int64_t stride, int64_t lim, float2 (&h)[2], float2 (&l)[2]) const {
+        if (amp_fp32) hops2_df_t<true>(tab, tstride, base, off, stride, lim, h, l);
+        else hops2_df_t<false>(tab, tstride, base, off, stride, lim, h, l);
+    }
+    template <bool kAmp32>
+    __device__ __forceinline__ void hops2_df_t(const int32_t* tab, int64_t tstride, const float4* base, int64_t off,
+                                               int64_t stride, int64_t lim, float2 (&h)[2], float2 (&l)[2]) const {
+        constexpr int kG = SCOCG_H2_GROUP;
+        for (int j0 = 0; j0 < S2; j0 += kG) {
+            int e[kG];
+            float4 xa[kG], xb[kG];
+            float th[kG], tl[kG];
+#pragma unroll
+            for (int q = 0; q < kG; ++q) {
+                e[q] = j0 + q < S2 ? tab[(int64_t)(j0 + q) * tstride] : -1;
+                if (e[q] >= 0 && !chk(dbg, 22, e[q] >> 8, lim)) e[q] = -1;
+            }
+#pragma unroll
+            for (int q = 0; q < kG; ++q) {
+                const float4* p = base + (int64_t)(max(e[q], 0) >> 8) * stride;
+                xa[q] = p[0];
+                xb[q] = p[off];
+                const float* t = reinterpret_cast<const float*>(ampf + (max(e[q], 0) & 255));
+                th[q] = t[0];
+                tl[q] = kAmp32 ? 0.f : t[2];
+            }
+#pragma unroll
+            for (int q = 0; q < kG; ++q) {
+                const float2 v = e[q] >= 0 ? make_float2(th[q], th[q]) : make_float2(0.f, 0.f);
+                if constexpr (kAmp32) {
+                    pk_acc_fx2(h[0], l[0], v, hi2(xa[q]), lo2(xa[q]));
+                    pk_acc_fx2(h[1], l[1], v, hi2(xb[q]), lo2(xb[q]));
+                } else {
+                    const float2 w = e[q] >= 0 ? make_float2(tl[q], tl[q]) : make_float2(0.f, 0.f);
+                    pk_acc_prod(h[0], l[0], v, w, hi2(xa[q]), lo2(xa[q]));
+                    pk_acc_prod(h[1], l[1], v, w, hi2(xb[q]), lo2(xb[q]));
+                }
+            }
+            if (e[kG - 1] < 0) break;
+        }
+    }
+    __device__ __forceinline__ void pass1(int64_t unit, int lane, float4 zs, float4 bp, const float4* x,
+                                          float4* q) const {
+        int u, d;
+        rc1(unit, lane, u, d);
+        if (d >= D_dn) return;
+        const bool two = u + 1 < D_up;
+        float2 h[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, l[2] = {h[0], h[0]};
+        hops2_df(hop_dn + d, D_dn, x + (size_t)u * D_dn, two ? D_dn : 0, 1, D_dn, h, l);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            if (k == 1 && !two) break;
+            const int64_t row = (int64_t)(u + k) * D_dn + d;
+            int cu, cp, cv;
+            counts(st_up[u + k], st_dn[d], u + k, d, cu, cp, cv);
+            float2 hj = make_float2(0.f, 0.f), lj = hj, hp = hj, lp = hj;
+            joint_df(u + k, d, x, hj, lj, hp, lp);
+            const float4 w = combine_df(u + k, d, cu, cp, cv, zs, x[row], h[k], l[k], hj, lj, hp, lp);
+            q[row] = vcfma(bp, q[row], w);
+        }
+    }
+    // on_row(row, q_n of the row) for each row of the unit
+    template <typename F>
+    __device__ __forceinline__ void pass2(int64_t unit, int lane, const float4* x, float4* q, F&& on_row) const {
+        int u, d;
+        rc2(unit, lane, u, d);
+        if (d >= D_dn) return;
+        const bool two = d + 32 < D_dn;
+        float2 h[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, l[2] = {h[0], h[0]};
+        hops2_df(hop_up + u, D_up, x + d, two ? 32 : 0, D_dn, D_up, h, l);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            if (k == 1 && !two) break;
+            const int64_t row = (int64_t)u * D_dn + d + 32 * k;
+            pk_norm(h[k], l[k]);
+            const float4 q1 = q[row];
+            float2 s, e;
+            pk_two_sum(hi2(q1), pk_neg(h[k]), s, e);
+            e = pk_add(e, pk_sub(lo2(q1), l[k]));
+            pk_norm(s, e);
+            const float4 qn = pk4(s, e);
+            q[row] = qn;
+            on_row(row, qn);
+        }
+    }
     // the row whose term (unit, lane) adds to the r^T q partial of phase A
     // (the tile-major order of the one-pass apply and of pass 2)
     __device__ __forceinline__ bool row_of(int64_t unit, int lane, int64_t& row) const {
@@ -276,41 +410,6 @@ struct ApplyHubbard2 {
         u = (int)((uint32_t)unit % (uint32_t)D_up);
         d = (int)((uint32_t)unit / (uint32_t)D_up) * 32 + lane;
         return d < D_dn;
-    }
-    __device__ __forceinline__ float4 pass1_w(int u, int d, float4 zs, const float4* x) const {
-        const int64_t row = (int64_t)u * D_dn + d;
-        const uint32_t su = st_up[u], sd = st_dn[d];
-        int cu, cp, cv;
-        counts(su, sd, u, d, cu, cp, cv);
-        float2 h = make_float2(0.f, 0.f), l = make_float2(0.f, 0.f);
-        hops_df(hop_dn + d, D_dn, x + (size_t)u * D_dn, 1, D_dn, h, l);
-        float2 hj = make_float2(0.f, 0.f), lj = hj, hp = hj, lp = hj;
-        joint_df(u, d, x, hj, lj, hp, lp);
-        return combine_df(u, d, cu, cp, cv, zs, x[row], h, l, hj, lj, hp, lp);
-    }
-    __device__ __forceinline__ void pass1(int64_t unit, int lane, float4 zs, float4 bp, const float4* x,
-                                          float4* q) const {
-        int u, d;
-        if (!rc_rows(unit, lane, u, d)) return;
-        const int64_t row = (int64_t)u * D_dn + d;
-        q[row] = vcfma(bp, q[row], pass1_w(u, d, zs, x));
-    }
-    __device__ __forceinline__ bool pass2(int64_t unit, int lane, const float4* x, float4* q, int64_t& row,
-                                          float4& qn) const {
-        int u, d;
-        if (!rc_tiles(unit, lane, u, d)) return false;
-        row = (int64_t)u * D_dn + d;
-        float2 h = make_float2(0.f, 0.f), l = make_float2(0.f, 0.f);
-        hops_df(hop_up + u, D_up, x + d, D_dn, D_up, h, l);
-        pk_norm(h, l);
-        const float4 q1 = q[row];
-        float2 s, e;
-        pk_two_sum(hi2(q1), pk_neg(h), s, e);
-        e = pk_add(e, pk_sub(lo2(q1), l));
-        pk_norm(s, e);
-        qn = pk4(s, e);
-        q[row] = qn;
-        return true;
     }
     // FP64 (double2) and complex64 (float2) vectors
     template <typename VV>
@@ -332,9 +431,15 @@ struct ApplyHubbard2 {
     }
     template <typename VV>
     __device__ __forceinline__ void pass1(int64_t unit, int lane, VV zs, VV bp, const VV* x, VV* q) const {
-        using T = decltype(zs.x);
         int u, d;
-        if (!rc_rows(unit, lane, u, d)) return;
+        rc1(unit, lane, u, d);
+        if (d >= D_dn) return;
+        pass1_row(u, d, zs, bp, x, q);
+        if (u + 1 < D_up) pass1_row(u + 1, d, zs, bp, x, q);
+    }
+    template <typename VV>
+    __device__ __forceinline__ void pass1_row(int u, int d, VV zs, VV bp, const VV* x, VV* q) const {
+        using T = decltype(zs.x);
         const int64_t row = (int64_t)u * D_dn + d;
         const uint32_t su = st_up[u], sd = st_dn[d];
         int cu, cp, cv;
@@ -358,16 +463,20 @@ struct ApplyHubbard2 {
         }
         q[row] = vcfma(bp, q[row], acc);
     }
-    template <typename VV>
-    __device__ __forceinline__ bool pass2(int64_t unit, int lane, const VV* x, VV* q, int64_t& row, VV& qn) const {
-        int u, d;
-        if (!rc_tiles(unit, lane, u, d)) return false;
-        row = (int64_t)u * D_dn + d;
-        const VV hs = hops_v(hop_up + u, D_up, x + d, D_dn, D_up);
-        qn = q[row];
-        qn.x -= hs.x; qn.y -= hs.y;
-        q[row] = qn;
-        return true;
+    template <typename VV, typename F>
+    __device__ __forceinline__ void pass2(int64_t unit, int lane, const VV* x, VV* q, F&& on_row) const {
+        for (int k = 0; k < 2; ++k) {
+            int u, d;
+            rc2(unit, lane, u, d);
+            d += 32 * k;
+            if (d >= D_dn) return;
+            const int64_t row = (int64_t)u * D_dn + d;
+            const VV hs = hops_v(hop_up + u, D_up, x + d, D_dn, D_up);
+            VV qn = q[row];
+            qn.x -= hs.x; qn.y -= hs.y;
+            q[row] = qn;
+            on_row(row, qn);
+        }
     }
 
     template <typename VV>
@@ -437,6 +546,7 @@ static ApplyHubbard2<R> make_apply2(const Hubbard& hb) {
     ap.selff_dn = hb.d_self2f + D;
     ap.amp = hb.d_amp2;
     ap.ampf = reinterpret_cast<const float4*>(hb.d_amp2f);
+    ap.amp_fp32 = hb.amp2_fp32;
     ap.cross = hb.d_cross2;
     ap.crossf = hb.d_cross2f;
     ap.S2 = hb.S2; ap.ns = hb.ns; ap.D_up = hb.D_up; ap.D_dn = hb.D_dn;
@@ -631,6 +741,9 @@ extern "C" int scocg_create_hubbard2(scocg_handle* out, int n_sites, int n_bonds
         bonds[2 * b] = bond_i[b]; bonds[2 * b + 1] = bond_j[b];
         for (int q = 0; q < 4; ++q) amp[4 * b + q] = bond_t[4 * b + q];
     }
+    hb.amp2_fp32 = 1;
+    for (double v : amp)
+        if ((double)(float)v != v) hb.amp2_fp32 = 0;
     for (size_t q = 0; q < amp.size(); ++q)   // entry 2 q + sign bit: the amplitude times its sign
         for (int sg = 0; sg < 2; ++sg) {
             const double v = sg ? -amp[q] : amp[q];

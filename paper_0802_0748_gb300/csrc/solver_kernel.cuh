@@ -338,7 +338,7 @@ __device__ __forceinline__ void shift_update(const ShiftState& S, int k, const S
 }
 
 // Applies whose phase A runs in two passes (they declare kTwoPass and
-// provide pass1 / pass2, see ApplyHubbard).
+// provide units1 / pass1 and units2 / pass2, see ApplyHubbard2).
 template <class A, class = void>
 struct HasTwoPass : std::false_type {};
 template <class A>
@@ -542,9 +542,17 @@ __device__ __forceinline__ void resume_partials(const SolveArgs<R>& a, const App
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int wi = a.rstate->rotated != 0 ? rotated_place(warp) : warp;
     AT rq[2] = {};
-    for (int lu = wi; lu < sh.nloc; lu += kWarps) {
-        int64_t row;
-        if (ap.row_of(sh.unit(lu), lane, row)) acc_bil(rq[0], rq[1], a.r[row], sh.get(sh.place(lu, lane), row));
+    if constexpr (HasTwoPass<Apply>::value) {
+        for (int64_t u = sh.cta + (int64_t)sh.G * wi; u < ap.units2(); u += (int64_t)sh.G * kWarps)
+            for (int k = 0; k < Apply::kRows; ++k) {
+                int64_t row;
+                if (ap.row2_of(u, lane, k, row)) acc_bil(rq[0], rq[1], a.r[row], a.q[row]);
+            }
+    } else {
+        for (int lu = wi; lu < sh.nloc; lu += kWarps) {
+            int64_t row;
+            if (ap.row_of(sh.unit(lu), lane, row)) acc_bil(rq[0], rq[1], a.r[row], sh.get(sh.place(lu, lane), row));
+        }
     }
     const int act = __syncthreads_count(active);
     PartialOut o = out;
@@ -778,14 +786,14 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
             // and, when the rounds do not come out even, one unit fewer
             const int wi = c_here ? rotated_place(warp) : warp;
             if constexpr (HasTwoPass<Apply>::value) {
-                // two passes over the units in two orders, a grid barrier between
-                for (int lu = wi; lu < sh.nloc; lu += kWarps) ap.pass1(sh.unit(lu), lane, s_vs[0], s_vs[1], (const V*)a.r, a.q);
+                // two passes over units of two rows a lane in two orders, a grid
+                // barrier between
+                const int64_t n1 = ap.units1(), n2 = ap.units2(), step = (int64_t)G * kWarps;
+                for (int64_t u = cta + (int64_t)G * wi; u < n1; u += step) ap.pass1(u, lane, s_vs[0], s_vs[1], (const V*)a.r, a.q);
                 if (!grid_barrier(a.sync, epoch)) return;
-                for (int lu = wi; lu < sh.nloc; lu += kWarps) {
-                    int64_t row;
-                    V qn;
-                    if (ap.pass2(sh.unit(lu), lane, (const V*)a.r, a.q, row, qn)) acc_bil(rq[0], rq[1], a.r[row], qn);
-                }
+                for (int64_t u = cta + (int64_t)G * wi; u < n2; u += step)
+                    ap.pass2(u, lane, (const V*)a.r, a.q,
+                             [&](int64_t row, V qn) { acc_bil(rq[0], rq[1], a.r[row], qn); });
             } else {
                 for (int lu = wi; lu < sh.nloc; lu += kWarps) {
                     int64_t row;
