@@ -731,8 +731,8 @@ __device__ __forceinline__ void stage_tri(const double* alpha, const double* bet
 }
 
 // Lowest eigenpair of the k x k tridiagonal T (alpha on the diagonal, beta
-// off it), one warp (80 steps: 735 us before the recurrences lost their divisions
-// and FP64 comparisons): multisection on the Sturm count (negative pivots of the
+// off it), one warp (the iterate in shared memory, elementwise divisions by all lanes, Sturm
+// tests on integers; 80 steps took 735 us before): multisection on the Sturm count (negative pivots of the
 // LDL^T factorisation of T - x) inside the Gershgorin interval, 32 points per
 // round, each lane counting at one point; then, in lane 0, three steps of
 // inverse iteration with T - theta factorised by Gaussian elimination with
@@ -774,8 +774,8 @@ __global__ void k_tri_lowest(const int* kdim, const double* alpha, const double*
         else { hi = xf; if (f > 0) lo = xp; }
     }
     const double th = 0.5 * (lo + hi);
-    // LU of T - th with row interchanges: U0 reciprocals of the diagonal, U1, U2
-    // superdiagonals, l multipliers, sw = 1 where rows i and i + 1 were exchanged
+    // LU of T - th with row interchanges: U0 diagonal, U1, U2 superdiagonals,
+    // l multipliers, sw = 1 where rows i and i + 1 were exchanged
     double* U0 = work;
     double* U1 = work + k;
     double* U2 = work + 2 * k;
@@ -802,8 +802,6 @@ __global__ void k_tri_lowest(const int* kdim, const double* alpha, const double*
         }
         U0[k - 1] = fabs(r0) < tiny ? (r0 < 0.0 ? -tiny : tiny) : r0;
     }
-    __syncwarp();
-    for (int i = lane; i < k; i += 32) U0[i] = 1.0 / U0[i];
     // the iterate in shared memory (the Sturm counts are done with s_b2)
     double* v = s_b2;
     __syncwarp();
@@ -824,7 +822,7 @@ __global__ void k_tri_lowest(const int* kdim, const double* alpha, const double*
                 double t = v[i];
                 if (i + 1 < k) t -= U1[i] * v1;
                 if (i + 2 < k) t -= U2[i] * v2;
-                t *= U0[i];
+                t /= U0[i];
                 v[i] = t;
                 v2 = v1; v1 = t;
             }
@@ -835,11 +833,13 @@ __global__ void k_tri_lowest(const int* kdim, const double* alpha, const double*
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         if (!(mx > 0.0) || !isfinite(mx)) break;
-        const double imx = 1.0 / mx;
-        double nr = 0.0;
-        for (int i = lane; i < k; i += 32) { const double t = v[i] * imx; v[i] = t; nr = fma(t, t, nr); }
-        const double inr = 1.0 / sqrt(warp_sum(nr));
-        for (int i = lane; i < k; i += 32) v[i] *= inr;
+        for (int i = lane; i < k; i += 32) v[i] /= mx;
+        __syncwarp();
+        double nr = 0.0;   // in every lane, in index order (the sign of s, and with it psi's, follows from rounding here)
+        for (int i = 0; i < k; ++i) nr += v[i] * v[i];
+        nr = sqrt(nr);
+        __syncwarp();
+        for (int i = lane; i < k; i += 32) v[i] /= nr;
     }
     __syncwarp();
     for (int i = lane; i < k; i += 32) s[i] = v[i];
