@@ -25,9 +25,6 @@
 #include "vector_ops.cuh"
 #include "hubbard_basis.cuh"
 
-#ifndef SCOCG_HOP_GROUP
-#define SCOCG_HOP_GROUP 4
-#endif
 
 namespace scocg {
 
@@ -68,6 +65,19 @@ __global__ void k_hubbard_tables(int L, int k, int D, int ring, uint32_t* states
     }
 }
 
+// four consecutive entries of a rank's hop list (past its S entries: -1); with S
+// a multiple of four (L even) each list starts on a 16-byte boundary and they are
+// one load, a quarter of the L1 wavefronts of a warp's 32 lists
+__device__ __forceinline__ void hop4(const int32_t* tab, int j0, int S, int (&e)[4]) {
+    if ((S & 3) == 0) {
+        const int4 v = *reinterpret_cast<const int4*>(tab + j0);
+        e[0] = v.x; e[1] = v.y; e[2] = v.z; e[3] = v.w;
+    } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) e[q] = j0 + q < S ? tab[j0 + q] : -1;
+    }
+}
+
 template <typename R>
 struct ApplyHubbard {
     static constexpr int kRowsPerUnit = 32;
@@ -94,16 +104,15 @@ struct ApplyHubbard {
     // taken as float pairs (exact for values such as t = 1, U = 4, V = 1).  The
     // hop lists are read kHopGroup entries at a time: the table entries, then
     // their gathers, are issued together (each list ends at its first -1).
-    static constexpr int kHopGroup = SCOCG_HOP_GROUP;
+    static constexpr int kHopGroup = 4;
     __device__ __forceinline__ static void hop_acc_df(const int32_t* tab, int S, const float4* base, int64_t stride,
                                                       int64_t lim, unsigned long long* dbg, float2& h, float2& l) {
         for (int j0 = 0; j0 < S; j0 += kHopGroup) {
             int e[kHopGroup];
+            hop4(tab, j0, S, e);
 #pragma unroll
-            for (int q = 0; q < kHopGroup; ++q) {
-                e[q] = j0 + q < S ? tab[j0 + q] : -1;
+            for (int q = 0; q < kHopGroup; ++q)
                 if (e[q] >= 0 && !chk(dbg, 20, e[q] >> 1, lim)) e[q] = -1;
-            }
             float4 xv[kHopGroup];
 #pragma unroll
             for (int q = 0; q < kHopGroup; ++q) xv[q] = base[(int64_t)(max(e[q], 0) >> 1) * stride];   // entry 0 when ended
@@ -294,8 +303,7 @@ __device__ __forceinline__ double hop_sum(const int32_t* tab, int S, const doubl
     for (int j0 = 0; j0 < S; j0 += kHopBatch) {
         int e[kHopBatch];
         double xv[kHopBatch];
-#pragma unroll
-        for (int q = 0; q < kHopBatch; ++q) e[q] = j0 + q < S ? tab[j0 + q] : -1;
+        hop4(tab, j0, S, e);
 #pragma unroll
         for (int q = 0; q < kHopBatch; ++q)
             if (e[q] >= 0) xv[q] = base[(int64_t)(e[q] >> 1) * stride];
