@@ -75,7 +75,7 @@ struct Hubbard {
     double Up = 0, J = 0, Jp = 0;
     int32_t* d_hop2 = nullptr;         // [2][Dmax][S2]: (target << 8) | (amplitude << 1) | (sign < 0), -1 = unused
     int32_t* d_orb2 = nullptr;         // [2][Dmax][ns]: (target << 1) | destination orbital, -1 = no move
-    uint32_t* d_nib2 = nullptr;        // [2][Dmax][2]: site occupations n_i and (A n)_i as nibbles
+    uint32_t* d_nib2 = nullptr;        // [2][Dmax][2]: site occupations n_i and (A n)_i as nibbles; more than 8 sites: twice
     double* d_self2 = nullptr;         // [2][Dmax]: the diagonal terms of one spin alone
     float2* d_self2f = nullptr;        // [2][Dmax]: the same as float pairs (hi, lo)
     double* d_amp2 = nullptr;          // [nb][2][2] hoppings t_ab of each bond

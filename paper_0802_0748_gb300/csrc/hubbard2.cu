@@ -44,16 +44,13 @@ constexpr int kCross2 = 257;         // counts 0..256 of the cross-spin diagonal
 #define SCOCG_H2_GROUP 2   // hop entries of two rows read (and gathered) together
 #endif
 constexpr int kHop2Group = 4;   // the same of one row
-#ifndef SCOCG_H2_UMAJOR
-#define SCOCG_H2_UMAJOR 0
-#endif
 
 __device__ __forceinline__ int parity_sign(int c) { return (c & 1) ? -1 : 1; }
 
 // One thread per rank of one spin species: the basis string, the hop list, the
 // orbital-move list and the spin's own diagonal terms.
 __global__ void k_hubbard2_tables(int ns, int nb, int k, int D, const int32_t* bonds, double Up, double J, double V,
-                                  int S2, uint32_t* states, int32_t* hop, int32_t* orb, uint32_t* nib, double* self,
+                                  int S2, uint32_t* states, int32_t* hop, int32_t* orb, uint32_t* nib, uint32_t* nib_hi, double* self,
                                   float2* selff) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= D) return;
@@ -78,7 +75,7 @@ __global__ void k_hubbard2_tables(int ns, int nb, int k, int D, const int32_t* b
             }
     }
     for (int c = cnt; c < S2; ++c) hop[(size_t)c * D + r] = -1;
-    uint32_t ni = 0, ani = 0;
+    uint64_t ni = 0, ani = 0;
     double sv = 0.0;
     int same = 0;
     for (int i = 0; i < ns; ++i) {
@@ -89,18 +86,22 @@ __global__ void k_hubbard2_tables(int ns, int nb, int k, int D, const int32_t* b
             mv = (int32_t)(rank_of(s ^ (3u << (2 * i))) << 1) | dst;
         }
         orb[(size_t)i * D + r] = mv;
-        ni |= (uint32_t)__popc(o) << (4 * i);
+        ni |= (uint64_t)__popc(o) << (4 * i);
         same += o == 3u;
     }
     for (int b = 0; b < nb; ++b) {
         const int i = bonds[2 * b], j = bonds[2 * b + 1];
-        const uint32_t n_i = (ni >> (4 * i)) & 15u, n_j = (ni >> (4 * j)) & 15u;
+        const uint32_t n_i = (uint32_t)(ni >> (4 * i)) & 15u, n_j = (uint32_t)(ni >> (4 * j)) & 15u;
         sv += (double)(n_i * n_j);
-        ani += n_j << (4 * i);
-        ani += n_i << (4 * j);
+        ani += (uint64_t)n_j << (4 * i);
+        ani += (uint64_t)n_i << (4 * j);
     }
-    nib[2 * (size_t)r] = ni;
-    nib[2 * (size_t)r + 1] = ani;
+    nib[2 * (size_t)r] = (uint32_t)ni;
+    nib[2 * (size_t)r + 1] = (uint32_t)ani;
+    if (ns > 8) {
+        nib_hi[2 * (size_t)r] = (uint32_t)(ni >> 32);
+        nib_hi[2 * (size_t)r + 1] = (uint32_t)(ani >> 32);
+    }
     const double d = (Up - J) * (double)same + V * sv;
     self[r] = d;
     const float hi = (float)d;
@@ -118,7 +119,9 @@ struct ApplyHubbard2 {
     const int32_t* orb_up;
     const int32_t* orb_dn;     // [ns][D]
     const uint32_t* nib_up;
-    const uint32_t* nib_dn;    // [D][2]
+    const uint32_t* nib_dn;    // [D][2], sites 0..7
+    const uint32_t* nibh_up;   // the same of sites 8..15 (read when ns > 8)
+    const uint32_t* nibh_dn;
     const double* self_up;
     const double* self_dn;
     const float2* selff_up;
@@ -135,18 +138,17 @@ struct ApplyHubbard2 {
     unsigned long long* dbg;
 
     // Row (u, d) of (unit, lane).  Units are visited by all CTAs together in
-    // unit order; up-major (unit = u * tiles + tile) keeps the rows x[u][:] of
-    // the down hops and the joint moves' rows in cache, tile-major (unit =
-    // tile * D_up + u) the column tiles x[:][tile] of the up hops.
+    // tile-major order (unit = tile * D_up + u), which keeps the column tiles
+    // x[:][tile] of the up hops in cache.
     __device__ __forceinline__ void unit_rc(int64_t unit, int lane, int& u, int& d) const {
-#if SCOCG_H2_UMAJOR
-        const int tiles = (D_dn + 31) / 32;
-        u = (int)((uint32_t)unit / (uint32_t)tiles);
-        d = (int)((uint32_t)unit % (uint32_t)tiles) * 32 + lane;
-#else
         u = (int)((uint32_t)unit % (uint32_t)D_up);
         d = (int)((uint32_t)unit / (uint32_t)D_up) * 32 + lane;
-#endif
+    }
+
+    // sum_i n_i (A n)_i over eight sites' nibbles, as two packed byte products
+    static __device__ __forceinline__ int cross_sum(uint32_t n, uint32_t an) {
+        constexpr uint32_t kNib = 0x0f0f0f0fu;
+        return (int)__dp4a(n & kNib, an & kNib, __dp4a((n >> 4) & kNib, (an >> 4) & kNib, 0u));
     }
 
     // the cross-spin diagonal counts of row (u, d)
@@ -154,16 +156,8 @@ struct ApplyHubbard2 {
         const uint32_t ev = 0x55555555u;
         cu = __popc(su & sd);
         cp = __popc(su & (sd >> 1) & ev) + __popc(sd & (su >> 1) & ev);
-        const uint32_t nu = nib_up[2 * (size_t)u], and_ = nib_dn[2 * (size_t)d + 1];
-        int c = 0;
-        if (ns <= 8) {   // eight sites' nibbles as two packed byte products
-            constexpr uint32_t kNib = 0x0f0f0f0fu;
-            c = (int)__dp4a(nu & kNib, and_ & kNib, __dp4a((nu >> 4) & kNib, (and_ >> 4) & kNib, 0u));
-        } else {
-#pragma unroll 4
-            for (int i = 0; i < ns; ++i) c += (int)(((nu >> (4 * i)) & 15u) * ((and_ >> (4 * i)) & 15u));
-        }
-        cv = c;
+        cv = cross_sum(nib_up[2 * (size_t)u], nib_dn[2 * (size_t)d + 1]);
+        if (ns > 8) cv += cross_sum(nibh_up[2 * (size_t)u], nibh_dn[2 * (size_t)d + 1]);
     }
 
     // Compensated vectors: per hop a product of the amplitude (float pair)
@@ -540,6 +534,8 @@ static ApplyHubbard2<R> make_apply2(const Hubbard& hb) {
     ap.orb_dn = hb.d_orb2 + D * hb.ns;
     ap.nib_up = hb.d_nib2;
     ap.nib_dn = hb.d_nib2 + 2 * D;
+    ap.nibh_up = hb.d_nib2 + 4 * D;
+    ap.nibh_dn = hb.d_nib2 + 6 * D;
     ap.self_up = hb.d_self2;
     ap.self_dn = hb.d_self2 + D;
     ap.selff_up = hb.d_self2f;
@@ -762,7 +758,8 @@ extern "C" int scocg_create_hubbard2(scocg_handle* out, int n_sites, int n_bonds
     cudaError_t e = cudaMalloc(&hb.d_states, sizeof(uint32_t) * 2 * D);
     if (e == cudaSuccess) e = cudaMalloc(&hb.d_hop2, sizeof(int32_t) * 2 * D * hb.S2);
     if (e == cudaSuccess) e = cudaMalloc(&hb.d_orb2, sizeof(int32_t) * 2 * D * n_sites);
-    if (e == cudaSuccess) e = cudaMalloc(&hb.d_nib2, sizeof(uint32_t) * 2 * D * 2);
+    const size_t nib_words = n_sites > 8 ? 8 * D : 4 * D;
+    if (e == cudaSuccess) e = cudaMalloc(&hb.d_nib2, sizeof(uint32_t) * nib_words);
     if (e == cudaSuccess) e = cudaMalloc(&hb.d_self2, sizeof(double) * 2 * D);
     if (e == cudaSuccess) e = cudaMalloc(&hb.d_self2f, sizeof(float2) * 2 * D);
     if (e == cudaSuccess) e = cudaMalloc(&hb.d_amp2, sizeof(double) * amp.size());
@@ -779,12 +776,12 @@ extern "C" int scocg_create_hubbard2(scocg_handle* out, int n_sites, int n_bonds
         const int Ds = sp ? hb.D_dn : hb.D_up, k = sp ? n_dn : n_up;
         k_hubbard2_tables<<<(Ds + 127) / 128, 128, 0, s>>>(n_sites, n_bonds, k, Ds, hb.d_bonds2, Up, J, V, hb.S2,
                                                            hb.d_states + sp * D, hb.d_hop2 + sp * D * hb.S2,
-                                                           hb.d_orb2 + sp * D * n_sites, hb.d_nib2 + sp * D * 2,
+                                                           hb.d_orb2 + sp * D * n_sites, hb.d_nib2 + sp * D * 2, hb.d_nib2 + (n_sites > 8 ? 4 * D : 0) + sp * D * 2,
                                                            hb.d_self2 + sp * D, hb.d_self2f + sp * D);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    hb.table_bytes = (double)(hb.D_up + hb.D_dn) * (4.0 + 4.0 * hb.S2 + 4.0 * n_sites + 8.0 + 8.0);
+    hb.table_bytes = (double)(hb.D_up + hb.D_dn) * (4.0 + 4.0 * hb.S2 + 4.0 * n_sites + (n_sites > 8 ? 16.0 : 8.0) + 8.0);
     if (e != cudaSuccess) { st = cuda_status(e); h->free_all(); delete h; return st; }
     *out = h;
     return SCOCG_OK;
