@@ -49,6 +49,70 @@ def shift_grid(K):
     return np.linspace(-3.0, 3.0, K) + 0.1j
 
 
+# Grids of one CTA, around the two reductions' limit (32 CTAs: packets up to it,
+# the counter barrier above) and beyond the units of work (the largest is
+# clamped); 70 shifts give a CTA 70 of them (too many to keep), 24, 3, 3, 2 and
+# fewer; 1 and 2 projections keep the shift scalars on the chip, 3 do not.
+@pytest.mark.parametrize("prec,bound", [(0, 1e-10), (2, 1e-9), (1, 5e-4)])
+@pytest.mark.parametrize("grid", [0, 1, 3, 31, 32, 33, 152])
+@pytest.mark.parametrize("kind", ["blocks", "scalar"])
+def test_solve_over_grids(S, kind, grid, prec, bound):
+    h_csr = inputs.anderson_csr(6, seed=11) if kind == "blocks" else inputs.chain_csr(1037, t=-0.9)
+    n = h_csr.n
+    b = inputs.random_unit_complex(n, 3)
+    H = h_csr.dense()
+    e, U = np.linalg.eigh(H.astype(np.float32).astype(np.float64) if prec else H)   # H as the mode holds it
+    h = S.scocg_create_csr(h_csr.rowptr, h_csr.col, h_csr.val, opts=S.SolveOptions(precision=prec, grid=grid))
+    try:
+        for K, M in ((70, 1), (70, 3), (33, 2), (1, 1)):
+            z = shift_grid(K)
+            idx = [0, n - 1, n // 2][:M]
+            G, info = S.scocg_solve(h, z, cuda(b), proj_idx=idx, tol=1e-5 if prec == 1 else 1e-12)
+            assert info["status"] == 0
+            want = np.einsum("mi,ki,i->mk", U[idx], 1.0 / (z[:, None] - e[None, :]), U.T @ b)
+            got = G.cpu().numpy()[0]
+            assert got.shape == want.shape
+            assert np.max(np.abs(got - want)) <= bound, (K, M)
+    finally:
+        S.scocg_destroy(h)
+
+
+# Full-vector items are (32 rows, a shift): one row, a ragged last chunk, odd
+# numbers of shifts, one CTA and the default grid.
+@pytest.mark.parametrize("grid", [0, 1])
+@pytest.mark.parametrize("n,K", [(1, 3), (31, 1), (33, 7), (500, 5), (1037, 33)])
+def test_full_vectors_ragged(S, n, K, grid):
+    h_csr = inputs.anderson_csr(5, seed=5) if n == 500 else inputs.chain_csr(n, t=-0.9, onsite=0.2)
+    assert h_csr.n == n
+    b = inputs.random_unit_complex(n, 7)
+    z = shift_grid(K)
+    h = S.scocg_create_csr(h_csr.rowptr, h_csr.col, h_csr.val, opts=S.SolveOptions(grid=grid))
+    try:
+        X, info = S.scocg_solve_full(h, z, cuda(b), tol=1e-12)
+    finally:
+        S.scocg_destroy(h)
+    assert info["status"] == 0
+    e, U = np.linalg.eigh(h_csr.dense())
+    want = ((U.T @ b)[None, :] / (z[:, None] - e[None, :])) @ U.T
+    assert np.max(np.abs(X.cpu().numpy().reshape(K, n) - want)) <= 1e-10
+
+
+# 608 eigenvalues: 32 lanes each on 152 SMs, 609: eight; the ends of both forms.
+@pytest.mark.parametrize("nu", [1, 2, 31, 608, 609, 1001])
+def test_tridiagonal_eigenvalues(S, nu):
+    h_csr = inputs.chain_csr(2048, t=-1.0)
+    b = np.zeros(h_csr.n)
+    b[0] = 1.0
+    h = S.scocg_create_csr(h_csr.rowptr, h_csr.col, h_csr.val)
+    try:
+        _, ritz, _, info = S.scocg_krylov_sd(h, cuda(b), nu, np.array([0.3 + 0.1j]), proj_idx=[0])
+    finally:
+        S.scocg_destroy(h)
+    assert info["nu_used"] == nu
+    ref = np.sort(-2.0 * np.cos(np.pi * np.arange(1, nu + 1) / (nu + 1)))
+    assert np.max(np.abs(ritz.cpu().numpy()[:nu] - ref)) < 1e-13
+
+
 # Rows in pairs: odd and even numbers of up states (15, 20, 6) against ragged
 # tiles of 64 down states; 9 sites take the general cross-spin counts.  Values
 # in FP32 (exact amplitudes) and not.
@@ -80,5 +144,26 @@ def test_two_orbital_rows(S, oracle_mod, sites, nu, nd, fp32):
         assert np.max(np.abs(y32 - want)) <= 1e-5 * scale
         ydf = from_df(S.scocg_apply(h, z, cuda(to_df(x)), precision=S.MIXED_DF).cpu().numpy())
         assert np.max(np.abs(ydf - want)) <= 1e-12 * scale
+    finally:
+        S.scocg_destroy(h)
+
+
+# Hop lists of an even ring are read four entries at a time, of an odd one (or
+# an open chain's) singly; t, U, V and x are integers, so every form is exact.
+@pytest.mark.parametrize("periodic", [True, False])
+@pytest.mark.parametrize("L,nu,nd", [(3, 1, 2), (5, 2, 3), (6, 3, 3), (7, 3, 4), (8, 4, 4), (9, 4, 3)])
+def test_ring_hop_lists(S, oracle_mod, L, nu, nd, periodic):
+    import scipy.sparse as sp
+    rp, c, v = oracle_mod.hubbard_csr(L, nu, nd, 1.0, 4.0, 1.0, periodic)
+    n = rp.size - 1
+    H = sp.csr_matrix((v, c, rp), shape=(n, n))
+    rng = np.random.default_rng(L)
+    x = (rng.integers(-8, 9, n) + 1j * rng.integers(-8, 9, n)).astype(np.complex128)
+    z = 0.5 + 0.25j
+    want = z * x - H @ x
+    h = S.scocg_create_hubbard(L, nu, nd, 1.0, 4.0, 1.0, periodic)
+    try:
+        assert np.array_equal(S.scocg_apply(h, z, cuda(x)).cpu().numpy(), want)
+        assert np.array_equal(from_df(S.scocg_apply(h, z, cuda(to_df(x)), precision=S.MIXED_DF).cpu().numpy()), want)
     finally:
         S.scocg_destroy(h)
