@@ -159,9 +159,9 @@ struct ApplyHubbard {
         return true;
     }
 
-    // one pass per apply (the two-pass form of the two-orbital model measured
-    // slower here: 686 against 622 us per iteration at 14 sites)
-    // the row whose term (unit, lane) adds to the r^T q partial of phase A
+    // One pass per apply: the two-pass form of the two-orbital model measured
+    // slower here (686 against 622 us per iteration at 14 sites).
+    // row_of: the row whose term (unit, lane) adds to the r^T q partial of phase A
     __device__ __forceinline__ bool row_of(int64_t unit, int lane, int64_t& row) const {
         const int u = (int)((uint32_t)unit % (uint32_t)D_up), d = (int)((uint32_t)unit / (uint32_t)D_up) * 32 + lane;
         row = (int64_t)u * D_dn + d;
