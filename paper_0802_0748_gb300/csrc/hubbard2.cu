@@ -556,6 +556,12 @@ static ApplyHubbard2<R> make_apply2(const Hubbard& hb) {
 
 int hubbard2_max_ctas(const Hubbard& hb, int prec, int num_sms, size_t dyn_smem) {
     int nb = 0;
+    if (dyn_smem > 0) {   // above the 48 KB default together with the static part
+        const void* k = prec == SCOCG_MIXED      ? (const void*)cocg_persistent<float, ApplyHubbard2<float>>
+                        : prec == SCOCG_MIXED_DF ? (const void*)cocg_persistent<DF, ApplyHubbard2<float>>
+                                                 : (const void*)cocg_persistent<double, ApplyHubbard2<double>>;
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemMax);
+    }
     cudaError_t e =
         prec == SCOCG_MIXED
             ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, cocg_persistent<float, ApplyHubbard2<float>>, kBlock,
