@@ -72,13 +72,6 @@ __device__ __forceinline__ float2 pk_add(float2 a, float2 b) { return __fadd2_rn
 __device__ __forceinline__ float2 pk_sub(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
 __device__ __forceinline__ float2 pk_mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 pk_fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-// a rounded product that an addition follows: the assembler fuses a paired
-// multiply whose only use is a paired addition into one FMA (the sum's error
-// then loses the product's own rounding: 1.6e-8 instead of 3e-14 on 28-term
-// sums), which it does not do with the scalar multiply
-__device__ __forceinline__ float2 pk_mul_rn(float2 a, float2 b) {
-    return make_float2(__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y));
-}
 __device__ __forceinline__ float2 pk_neg(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.x, v.y); }
 __device__ __forceinline__ float2 lo2(float4 v) { return make_float2(v.z, v.w); }
@@ -97,10 +90,9 @@ __device__ __forceinline__ void pk_norm(float2& hi, float2& lo) {
     hi = s;
 }
 // (ah, al) += (xh + xl) * (yh + yl) lane by lane, the product exact to DF and
-// the sum by TwoSum, without renormalising the accumulator.  (Folding the
-// product's remainder into the TwoSum as below saves one instruction here but
-// rounds the low part twice more: the 64^3 x 4 solve at Im z = 1e-3 then took
-// more than 400,000 iterations instead of 120,000.)
+// the sum by TwoSum, without renormalising the accumulator.  (With the product's
+// remainder folded into the TwoSum, see pk_acc_fx2, the 64^3 x 4 solve at Im z =
+// 1e-3 took more than 400,000 iterations instead of 120,000.)
 __device__ __forceinline__ void pk_acc_prod(float2& ah, float2& al, float2 xh, float2 xl, float2 yh, float2 yl) {
     const float2 p = pk_mul(xh, yh);
     float2 e = pk_fma(xh, yh, pk_neg(p));
@@ -110,19 +102,20 @@ __device__ __forceinline__ void pk_acc_prod(float2& ah, float2& al, float2 xh, f
     ah = s;
     al = pk_add(al, pk_add(t, e));
 }
-// (ah, al) += v * (xh + xl) for an FP32 v, the apply's step.  With p the rounded
-// product and s = ah + p by TwoSum (bb = s - ah), the two exact remainders
-// (v xh - p) + (p - bb) are one fused operation, v xh - bb, rounded once: 21
-// cycles of a scheduler's FP32 pipe per warp (a paired add holds it two cycles,
-// a paired FMA 2.4) instead of 26 with TwoProd and TwoSum one after the other,
-// at the same error of a 28-term sum (rms 2.74e-15 against 2.70e-15 of the terms'
-// magnitude).  The apply's 28 steps per row are what that pipe spends most of its
-// time on.
+// (ah, al) += v * (xh + xl) for an FP32 v, the apply's step: TwoProd, TwoSum and
+// one addition of both remainders to the low part.  (Folding the two exact
+// remainders (v xh - p) + (p - bb) into one fused operation v xh - bb takes 21
+// instead of 26 cycles of a scheduler's FP32 pipe per warp, 57.7 against 61 us
+// per iteration at 64^3 x 4, but rounds at the size of the sum where this step
+// rounds at the product's: the error of a 7-term sum grows by 2.5 %, of 28 terms
+// by 2.0 %.)
 __device__ __forceinline__ void pk_acc_fx2(float2& ah, float2& al, float2 v, float2 xh, float2 xl) {
-    const float2 s = pk_add(ah, pk_mul_rn(v, xh)), bb = pk_sub(s, ah);
-    const float2 u = pk_add(pk_sub(ah, pk_sub(s, bb)), pk_fma(v, xh, pk_neg(bb)));
+    const float2 p = pk_mul(v, xh);
+    const float2 e = pk_fma(v, xl, pk_fma(v, xh, pk_neg(p)));
+    float2 s, t;
+    pk_two_sum(ah, p, s, t);
     ah = s;
-    al = pk_add(al, pk_fma(v, xl, u));
+    al = pk_add(al, pk_add(t, e));
 }
 
 // complex a * b + c: (re, im) += (a.re, a.re) (b.re, b.im) + (-a.im, a.im) (b.im, b.re)
