@@ -304,6 +304,25 @@ __device__ __forceinline__ ShiftState own_view(OwnShifts& o) {
     return ShiftState{o.pi_prev, o.pi_cur, o.sigma, o.alpha_k, o.inv_cur, o.P, o.X, o.frozen, o.iters, o.resid};
 }
 
+// pi_{n+1} = (1 + alpha sigma) pi_n + t2 (pi_n - pi_{n-1}), t2 = alpha_n beta_{n-1} /
+// alpha_{n-1}.  With the operations spelt out, so that every place that forms it
+// from the same inputs has the same bits: the full-vector mode's steps and the
+// recurrence would otherwise use different numbers wherever pi_{n+1} comes out of
+// a cancellation, and x^k loses what they differ by (t2 rounded in another order
+// there: errors of x 20 to 35 % larger at Im z = 0.1, up to 25 times on single systems).
+__device__ __forceinline__ double2 pi_next(double2 alpha, double2 t2, double2 sigma, double2 pc, double2 pp) {
+    const auto mul = [](double2 a, double2 b) {
+        return c2(fma(a.x, b.x, -__dmul_rn(a.y, b.y)), fma(a.x, b.y, __dmul_rn(a.y, b.x)));
+    };
+    const auto add = [](double2 a, double2 b) { return c2(__dadd_rn(a.x, b.x), __dadd_rn(a.y, b.y)); };
+    return add(mul(add(c2(1, 0), mul(alpha, sigma)), pc), mul(t2, add(pc, c2(-pp.x, -pp.y))));
+}
+
+// t2 from beta_{n-1} / alpha_{n-1}, which is known before alpha_n
+__device__ __forceinline__ double2 shift_t2(double2 alpha, double2 ratio) {
+    return c2(fma(alpha.x, ratio.x, -__dmul_rn(alpha.y, ratio.y)), fma(alpha.x, ratio.y, __dmul_rn(alpha.y, ratio.x)));
+}
+
 // Phase C for the shift in slot k of S: the pi three-term recurrence, the
 // projected p^k and x^k, the residual estimate and freezing.  Sets bad for a
 // zero or non-finite pi (its state is then left as it was), active when the
@@ -311,7 +330,7 @@ __device__ __forceinline__ ShiftState own_view(OwnShifts& o) {
 __device__ __forceinline__ void shift_update(const ShiftState& S, int k, const ShiftInputs& c, int M, double tol,
                                              double tol2, int& active, int& bad) {
     const double2 pp = S.pi_prev[k], pc = S.pi_cur[k], ic = S.inv_cur[k];
-    const double2 pn = cadd(cmul(cadd(c2(1, 0), cmul(c.alpha, S.sigma[k])), pc), cmul(c.t2, csub(pc, pp)));
+    const double2 pn = pi_next(c.alpha, c.t2, S.sigma[k], pc, pp);
     const double2 in = crecip(pn);
     const double2 ratio = cmul(pp, ic);                        // pi_{n-1} / pi_n
     const double2 beta_k = cmul(cmul(ratio, ratio), c.beta_prev);
@@ -864,7 +883,8 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
         }
 
         // ---- full-vector mode: this iteration's shift scalars for all shifts
-        // (every CTA computes them, with the same arithmetic as phase C).  The
+        // (every CTA computes them; t2, pi and its reciprocal bit for bit as phase
+        // C does, see pi_next).  The
         // directions are stored as pt^k = p^k / t_k with t_k = 1 / pi^k of the
         // iteration that wrote them, so that pt^k_n = r_n + cp pt^k_{n-1} and
         // x^k += cx pt^k take one complex FMA each:
@@ -877,14 +897,13 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
                 int* s_list = reinterpret_cast<int*>(s_full + 3 * a.K);   // the unconverged shifts, in any order
                 if (tid == 0) s_nact = 0;
                 __syncthreads();
-                const double2 t2 = cdiv(cmul(s.alpha, s.beta_prev), s.alpha_prev);
+                const double2 t2 = shift_t2(s.alpha, s.t2_ratio);   // phase C's, see pi_next
                 for (int k = tid; k < a.K; k += kBlock) {
                     if (__ldcg(a.S.frozen + k)) continue;
                     const double2 pp = __ldcg(a.S.pi_prev + k), pc = __ldcg(a.S.pi_cur + k);
                     const double2 ic = __ldcg(a.S.inv_cur + k);
                     const double2 ratio = cmul(pp, ic);
-                    const double2 pn = cadd(cmul(cadd(c2(1, 0), cmul(s.alpha, __ldcg(a.S.sigma + k))), pc),
-                                            cmul(t2, csub(pc, pp)));
+                    const double2 pn = pi_next(s.alpha, t2, __ldcg(a.S.sigma + k), pc, pp);
                     const double2 in = crecip(pn);
                     const double2 t = it == 0 ? c2(1, 0) : s_t[k];
                     s_cp[k] = cmul(cmul(cmul(cmul(ratio, ratio), s.beta_prev), pc), t);
@@ -1001,7 +1020,7 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
             s.cr_cur[tid] = s.cr_next[tid];
         }
         if (tid == 96) {
-            s_c.t2 = cmul(s.alpha, s.t2_ratio);
+            s_c.t2 = shift_t2(s.alpha, s.t2_ratio);
             s_c.alpha = s.alpha; s_c.beta_prev = s.beta_prev; s_c.n = it;
         } else if (tid == 32) {
             s_c.rn_b2 = s.red[2] * s.inv_b2;
