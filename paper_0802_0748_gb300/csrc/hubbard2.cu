@@ -269,32 +269,45 @@ struct ApplyHubbard2 {
     }
 
     // ---- two-pass form used by the persistent solve, kRows rows per lane and
-    // unit.  Pass 1 visits pairs of rows (u, u + 1) of a tile of 32 down ranks,
+    // unit.  Pass 1 visits kRows rows (u, u + 1) of a tile of 32 down ranks,
     // row-major (the CTAs share the rows x[u][:] of the down hops and the few rows
-    // of the joint moves): a lane's down-hop list and its amplitudes are read once
-    // for both rows.  It stores q = (z_s - diag) x - (down hops and joint moves) +
-    // beta q_old.  Pass 2 visits pairs of tiles of one row u, tile-major (the CTAs
-    // share the column tiles x[:][tile] of the up hops): the up-hop list serves 64
-    // down ranks; it subtracts the up hops.  (One row per lane spent as much on the
-    // lists as on the arithmetic: 3 up / 4 down of the 8-site cluster 165 us per
-    // iteration.)
+    // of the joint moves).  It stores q = (z_s - diag) x - (down hops and joint
+    // moves) + beta q_old.  Pass 2 visits kRows tiles of one row u, tile-major (the
+    // CTAs share the column tiles x[:][tile] of the up hops); it subtracts the up
+    // hops.  Compensated vectors take two rows: a lane's hop list and its amplitudes
+    // are read once for both, which one row per lane spent as much on as on the
+    // arithmetic (3 up / 4 down of the 8-site cluster, 128 shifts: 179 us per
+    // iteration with one row, 145 with two).  complex128 and complex64 vectors take
+    // one: two rows, one after the other, read the lists twice all the same and
+    // leave fewer units to share out (3 up / 3 down: complex64 71 us per iteration
+    // with one row, 93 with two; complex128 145 and 158).
     static constexpr bool kTwoPass = true;
-    static constexpr int kRows = 2;
-    __device__ __forceinline__ int64_t units1() const { return (int64_t)((D_up + 1) / 2) * ((D_dn + 31) / 32); }
-    __device__ __forceinline__ int64_t units2() const { return (int64_t)D_up * ((D_dn + 63) / 64); }
-    // rank pair of pass 1's and pass 2's units: row k is (u + k, d) or (u, d + 32 k)
+    template <typename VV>
+    static constexpr int kRows = std::is_same<VV, float4>::value ? 2 : 1;
+    template <typename VV>
+    __device__ __forceinline__ int64_t units1() const {
+        return (int64_t)((D_up + kRows<VV> - 1) / kRows<VV>) * ((D_dn + 31) / 32);
+    }
+    template <typename VV>
+    __device__ __forceinline__ int64_t units2() const {
+        return (int64_t)D_up * ((D_dn + 32 * kRows<VV> - 1) / (32 * kRows<VV>));
+    }
+    // ranks of pass 1's and pass 2's units: row k is (u + k, d) or (u, d + 32 k)
+    template <typename VV>
     __device__ __forceinline__ void rc1(int64_t unit, int lane, int& u, int& d) const {
         const uint32_t tiles = (uint32_t)(D_dn + 31) / 32;
-        u = 2 * (int)((uint32_t)unit / tiles);
+        u = kRows<VV> * (int)((uint32_t)unit / tiles);
         d = (int)((uint32_t)unit % tiles) * 32 + lane;
     }
+    template <typename VV>
     __device__ __forceinline__ void rc2(int64_t unit, int lane, int& u, int& d) const {
         u = (int)((uint32_t)unit % (uint32_t)D_up);
-        d = (int)((uint32_t)unit / (uint32_t)D_up) * 64 + lane;
+        d = (int)((uint32_t)unit / (uint32_t)D_up) * (32 * kRows<VV>) + lane;
     }
+    template <typename VV>
     __device__ __forceinline__ bool row2_of(int64_t unit, int lane, int k, int64_t& row) const {
         int u, d;
-        rc2(unit, lane, u, d);
+        rc2<VV>(unit, lane, u, d);
         row = (int64_t)u * D_dn + d + 32 * k;
         return d + 32 * k < D_dn;
     }
@@ -346,7 +359,7 @@ struct ApplyHubbard2 {
     __device__ __forceinline__ void pass1(int64_t unit, int lane, float4 zs, float4 bp, const float4* x,
                                           float4* q) const {
         int u, d;
-        rc1(unit, lane, u, d);
+        rc1<float4>(unit, lane, u, d);
         if (d >= D_dn) return;
         const bool two = u + 1 < D_up;
         float2 h[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, l[2] = {h[0], h[0]};
@@ -367,7 +380,7 @@ struct ApplyHubbard2 {
     template <typename F>
     __device__ __forceinline__ void pass2(int64_t unit, int lane, const float4* x, float4* q, F&& on_row) const {
         int u, d;
-        rc2(unit, lane, u, d);
+        rc2<float4>(unit, lane, u, d);
         if (d >= D_dn) return;
         const bool two = d + 32 < D_dn;
         float2 h[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, l[2] = {h[0], h[0]};
@@ -425,15 +438,10 @@ struct ApplyHubbard2 {
     }
     template <typename VV>
     __device__ __forceinline__ void pass1(int64_t unit, int lane, VV zs, VV bp, const VV* x, VV* q) const {
-        int u, d;
-        rc1(unit, lane, u, d);
-        if (d >= D_dn) return;
-        pass1_row(u, d, zs, bp, x, q);
-        if (u + 1 < D_up) pass1_row(u + 1, d, zs, bp, x, q);
-    }
-    template <typename VV>
-    __device__ __forceinline__ void pass1_row(int u, int d, VV zs, VV bp, const VV* x, VV* q) const {
         using T = decltype(zs.x);
+        int u, d;
+        rc1<VV>(unit, lane, u, d);
+        if (d >= D_dn) return;
         const int64_t row = (int64_t)u * D_dn + d;
         const uint32_t su = st_up[u], sd = st_dn[d];
         int cu, cp, cv;
@@ -459,18 +467,15 @@ struct ApplyHubbard2 {
     }
     template <typename VV, typename F>
     __device__ __forceinline__ void pass2(int64_t unit, int lane, const VV* x, VV* q, F&& on_row) const {
-        for (int k = 0; k < 2; ++k) {
-            int u, d;
-            rc2(unit, lane, u, d);
-            d += 32 * k;
-            if (d >= D_dn) return;
-            const int64_t row = (int64_t)u * D_dn + d;
-            const VV hs = hops_v(hop_up + u, D_up, x + d, D_dn, D_up);
-            VV qn = q[row];
-            qn.x -= hs.x; qn.y -= hs.y;
-            q[row] = qn;
-            on_row(row, qn);
-        }
+        int u, d;
+        rc2<VV>(unit, lane, u, d);
+        if (d >= D_dn) return;
+        const int64_t row = (int64_t)u * D_dn + d;
+        const VV hs = hops_v(hop_up + u, D_up, x + d, D_dn, D_up);
+        VV qn = q[row];
+        qn.x -= hs.x; qn.y -= hs.y;
+        q[row] = qn;
+        on_row(row, qn);
     }
 
     template <typename VV>

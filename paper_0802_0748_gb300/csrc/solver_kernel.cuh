@@ -562,10 +562,11 @@ __device__ __forceinline__ void resume_partials(const SolveArgs<R>& a, const App
     const int wi = a.rstate->rotated != 0 ? rotated_place(warp) : warp;
     AT rq[2] = {};
     if constexpr (HasTwoPass<Apply>::value) {
-        for (int64_t u = sh.cta + (int64_t)sh.G * wi; u < ap.units2(); u += (int64_t)sh.G * kWarps)
-            for (int k = 0; k < Apply::kRows; ++k) {
+        using V = typename Vec<R>::T;
+        for (int64_t u = sh.cta + (int64_t)sh.G * wi; u < ap.template units2<V>(); u += (int64_t)sh.G * kWarps)
+            for (int k = 0; k < Apply::template kRows<V>; ++k) {
                 int64_t row;
-                if (ap.row2_of(u, lane, k, row)) acc_bil(rq[0], rq[1], a.r[row], a.q[row]);
+                if (ap.template row2_of<V>(u, lane, k, row)) acc_bil(rq[0], rq[1], a.r[row], a.q[row]);
             }
     } else {
         for (int lu = wi; lu < sh.nloc; lu += kWarps) {
@@ -805,9 +806,8 @@ __device__ __forceinline__ void cocg_body(const SolveArgs<R>& a, const Apply& ap
             // and, when the rounds do not come out even, one unit fewer
             const int wi = c_here ? rotated_place(warp) : warp;
             if constexpr (HasTwoPass<Apply>::value) {
-                // two passes over units of two rows a lane in two orders, a grid
-                // barrier between
-                const int64_t n1 = ap.units1(), n2 = ap.units2(), step = (int64_t)G * kWarps;
+                // two passes over the units in two orders, a grid barrier between
+                const int64_t n1 = ap.template units1<V>(), n2 = ap.template units2<V>(), step = (int64_t)G * kWarps;
                 for (int64_t u = cta + (int64_t)G * wi; u < n1; u += step) ap.pass1(u, lane, s_vs[0], s_vs[1], (const V*)a.r, a.q);
                 if (!grid_barrier(a.sync, epoch)) return;
                 for (int64_t u = cta + (int64_t)G * wi; u < n2; u += step)
