@@ -23,7 +23,6 @@ __host__ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
 }
 __host__ __device__ __forceinline__ double2 cscale(double2 a, double s) { return c2(a.x * s, a.y * s); }
 __host__ __device__ __forceinline__ double cabs2(double2 a) { return a.x * a.x + a.y * a.y; }
-__host__ __device__ __forceinline__ double cabs_(double2 a) { return hypot(a.x, a.y); }
 // 2^-e / |bs|^2 for bs = 2^-e b, e the exponent of b's larger component (so
 // |bs|^2 lies in [1, 8) and neither overflows nor underflows).
 __host__ __device__ __forceinline__ double scaled_recip(double2 b, double2& bs) {

@@ -320,8 +320,9 @@ __device__ __forceinline__ double hop_sum(const int32_t* tab, int S, const doubl
 // (x_prev and beta optional), same unit order as the solver's apply, and the
 // block's partial of x^T y in part[blockIdx.x].  A launch whose *skip is set
 // does nothing.
-// 64 registers, four blocks per SM: 32 registers and eight blocks spill and
-// measured 16.0 instead of 16.7 ms at 12 sites, 5.1 instead of 4.8 at 10.
+// 64 registers, four blocks per SM.  32 registers and eight blocks spill: a ground
+// state of 200 applies takes 5.1 instead of 4.8 ms at 10 sites, 16.0 instead of 16.7 at
+// 12, 147 either way at 14; what one size gains is less than what the other loses.
 __global__ void __launch_bounds__(kVecBlock) k_hub_hx(ApplyHubbard<double> ap, int64_t nunits, const double* x,
                                                       double* y, const double* xprev, const double* beta,
                                                       double sigma, const int* skip, double* part, int n_up, int n_dn) {

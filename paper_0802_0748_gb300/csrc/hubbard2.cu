@@ -40,10 +40,11 @@ namespace scocg {
 constexpr int kMaxSites2 = 16;       // 2 ns <= 32 modes per spin
 constexpr int kMaxBonds2 = 32;       // amplitude index b*4 + a*2 + a' < 128 (7 bits)
 constexpr int kCross2 = 257;         // counts 0..256 of the cross-spin diagonal tables (8 per bond at most)
-#ifndef SCOCG_H2_GROUP
-#define SCOCG_H2_GROUP 2   // hop entries of two rows read (and gathered) together
-#endif
-constexpr int kHop2Group = 4;   // the same of one row
+// Hop entries read (and gathered) together, of one row and of two rows (compensated
+// solve, 3 up / 4 down: 149 us per iteration with one entry, 141 with two, 147 with
+// four), and sites whose joint moves are (one 141, two 141, four 147; 4 up / 4 down
+// 429, 422, 440).
+constexpr int kHop2Group = 4, kHop2Pair = 2, kJointGroup = 2;
 
 __device__ __forceinline__ int parity_sign(int c) { return (c & 1) ? -1 : 1; }
 
@@ -195,14 +196,11 @@ struct ApplyHubbard2 {
         }
     }
 
-    // joint moves (spin flip: J, pair hopping: J'), summed separately; four sites'
-    // moves, then their gathers, are in flight together
+    // joint moves (spin flip: J, pair hopping: J'), summed separately; kJointGroup
+    // sites' moves, then their gathers, are in flight together
     __device__ __forceinline__ void joint_df(int u, int d, const float4* x, float2& hj, float2& lj, float2& hp,
                                              float2& lp) const {
-#ifndef SCOCG_H2_JOINT
-#define SCOCG_H2_JOINT 2
-#endif
-        constexpr int kG = SCOCG_H2_JOINT;
+        constexpr int kG = kJointGroup;
         for (int i0 = 0; i0 < ns; i0 += kG) {
             int32_t mu[kG], md[kG];
             float4 xv[kG];
@@ -281,11 +279,11 @@ struct ApplyHubbard2 {
     // CTAs share the column tiles x[:][tile] of the up hops); it subtracts the up
     // hops.  Compensated vectors take two rows: a lane's hop list and its amplitudes
     // are read once for both, which one row per lane spent as much on as on the
-    // arithmetic (3 up / 4 down of the 8-site cluster, 128 shifts: 179 us per
-    // iteration with one row, 145 with two).  complex128 and complex64 vectors take
-    // one: two rows, one after the other, read the lists twice all the same and
-    // leave fewer units to share out (3 up / 3 down: complex64 71 us per iteration
-    // with one row, 93 with two; complex128 145 and 158).
+    // arithmetic (3 up / 4 down of the 8-site cluster, 128 shifts: 100 iterations 18.0
+    // ms before, 14.5 now).  complex128 and complex64 vectors take one: two rows, one
+    // after the other, read the lists twice all the same and leave fewer units to
+    // share out (3 up / 3 down, 100 iterations: complex64 7.1 ms with one row, 9.3
+    // with two; complex128 14.5 and 15.8).
     static constexpr bool kTwoPass = true;
     template <typename VV>
     static constexpr int kRows = std::is_same<VV, float4>::value ? 2 : 1;
@@ -327,7 +325,7 @@ struct ApplyHubbard2 {
     template <bool kAmp32>
     __device__ __forceinline__ void hops2_df_t(const int32_t* tab, int64_t tstride, const float4* base, int64_t off,
                                                int64_t stride, int64_t lim, float2 (&h)[2], float2 (&l)[2]) const {
-        constexpr int kG = SCOCG_H2_GROUP;
+        constexpr int kG = kHop2Pair;
         for (int j0 = 0; j0 < S2; j0 += kG) {
             int e[kG];
             float4 xa[kG], xb[kG];
@@ -405,13 +403,7 @@ struct ApplyHubbard2 {
             on_row(row, qn);
         }
     }
-    // the row whose term (unit, lane) adds to the r^T q partial of phase A
-    // (the tile-major order of the one-pass apply and of pass 2)
-    __device__ __forceinline__ bool row_of(int64_t unit, int lane, int64_t& row) const {
-        const int u = (int)((uint32_t)unit % (uint32_t)D_up), d = (int)((uint32_t)unit / (uint32_t)D_up) * 32 + lane;
-        row = (int64_t)u * D_dn + d;
-        return d < D_dn;
-    }
+    // the real operator's units: one row a lane, row-major (pass 1) and tile-major (pass 2)
     __device__ __forceinline__ bool rc_rows(int64_t unit, int lane, int& u, int& d) const {
         const int tiles = (D_dn + 31) / 32;
         u = (int)((uint32_t)unit / (uint32_t)tiles);

@@ -369,7 +369,7 @@ struct SolveArgs {
     int strideB;
     GridSync sync;
     // packets of the partial sums, [kPktVals][grid] (phase A 2, phase B 5), or
-    // null: grid barriers (more than kPktCtas CTAs or dense projections)
+    // null: grid barriers (more than kPktCtas CTAs or more than one dense projection)
     ulonglong2* pk;
     SolveStats* stats;
     double2* G;                // out [nproj][K] for this right-hand side
@@ -404,11 +404,11 @@ inline size_t solve_smem(const SolveArgs<R>& a, int grid) {
 // what can be co-resident, maxco).  An iteration has about 10 us of serial work
 // whatever the grid, so CTAs are added only while they shorten the phases: a
 // complex128 unit occupies a scheduler's FP64 pipe ~4 us, so four units (one per
-// scheduler) make a CTA; eight FP32 units do.  16^3 x 4 FP64 (512 units): 23.6 us
-// per iteration at 32 CTAs, 13.7 at 128; 22^3 x 4 FP64: 24.4 at 84, 17.9 at 152;
-// 8^3 x 4 (64 units) FP64 11.6 at 16, 12.9 at 64, compensated 11.1 at 8, 13.7 at
+// scheduler) make a CTA; eight FP32 units do.  16^3 x 4 FP64 (512 units): 22.6 us
+// per iteration at 32 CTAs, 12.8 at 128; 22^3 x 4 FP64: 22.9 at 84, 17.1 at 152;
+// 8^3 x 4 (64 units) FP64 11.7 at 16, 12.3 at 64, compensated 11.4 at 8, 12.5 at
 // 32.  One CTA per SM serves up to 24 units per SM (30^3 x 4 compensated, 22 per
-// SM: 20.1 at 152, 21.0 at 211, 19.9 at 304), above that every SM takes all it can.
+// SM: 16.2 at 152, 17.9 at 211, 16.6 at 304), above that every SM takes all it can.
 inline int64_t grid_want(int64_t units, bool fp64, int num_sms, int64_t maxco) {
     const int64_t per = fp64 ? 4 : 8;
     if (units > 24LL * num_sms) return maxco;
@@ -416,10 +416,7 @@ inline int64_t grid_want(int64_t units, bool fp64, int num_sms, int64_t maxco) {
 }
 // q is kept in shared memory while the CTAs of an SM hold at most this much of
 // it: the rest of the SM's 256 KB is the L1 that the gathers of the apply use.
-#ifndef SCOCG_Q_SMEM_PER_SM
-#define SCOCG_Q_SMEM_PER_SM (112 << 10)
-#endif
-constexpr size_t kQSmemPerSm = SCOCG_Q_SMEM_PER_SM;
+constexpr size_t kQSmemPerSm = 112 << 10;
 // Opt-in limit given to every solve kernel that uses dynamic shared memory: one
 // constant (the largest use: a CTA's q and 512 shifts of the full-vector mode),
 // so that solves in different threads cannot lower it under each other.

@@ -5,10 +5,11 @@
 
 namespace scocg {
 
-// Reductions of the standalone vector kernels (256-thread blocks): a block's
-// partial sum lands in part[blockIdx.x]; every consuming block adds the G
-// partials in the same fixed order, so all blocks see the same bit-identical
-// total without a separate reduction launch.
+// Reductions of 256-thread blocks: a block's partial sum lands in
+// part[blockIdx.x], and the G partials are added in one fixed order.  Separate
+// launches have the last block of the producing one add them (block_total); the
+// cooperative recursion and the projections add them where they are used
+// (sum_partials): every block that does sees the same bits.
 constexpr int kVecBlock = 256;
 
 __device__ __forceinline__ void block_partial(double v, double* part) {

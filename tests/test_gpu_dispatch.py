@@ -1,7 +1,9 @@
-"""Both sides of every rule that chooses a form of a kernel by size: the grid
+"""Both sides of the rules that choose a form of a kernel by size: the grid
 and with it the reduction between CTAs and the place of the shift scalars, the
 full-vector item loop, the lanes per eigenvalue of the tridiagonal bisection,
-and the row and hop-list forms of the matrix-free Hubbard operators.
+and single applies of the matrix-free Hubbard operators.  (The place of q is in
+test_gpu_waits.py, the Hubbard kernels that only solves and ground states run in
+test_gpu_hubbard_passes.py.)
 
 References: dense eigendecompositions, the oracle's CSR operators and closed
 forms.  Bounds: a residual of tol leaves |dG| <= tol / eta (unit b and c; eta
@@ -113,9 +115,9 @@ def test_tridiagonal_eigenvalues(S, nu):
     assert np.max(np.abs(ritz.cpu().numpy()[:nu] - ref)) < 1e-13
 
 
-# Rows in pairs: odd and even numbers of up states (15, 20, 6) against ragged
-# tiles of 64 down states; 9 sites take the general cross-spin counts.  Values
-# in FP32 (exact amplitudes) and not.
+# A single apply, one row per lane: odd and even numbers of up states (15, 20, 6)
+# against ragged tiles of 32 down states; 9 sites take the cross-spin counts'
+# second word.  Values in FP32 (exact amplitudes) and not.
 @pytest.mark.parametrize("fp32", [True, False])
 @pytest.mark.parametrize("sites,nu,nd", [(3, 2, 2), (3, 3, 4), (3, 6, 3), (3, 1, 0), (4, 3, 4), (4, 4, 2), (9, 2, 1), (9, 1, 2)])
 def test_two_orbital_rows(S, oracle_mod, sites, nu, nd, fp32):
@@ -148,8 +150,9 @@ def test_two_orbital_rows(S, oracle_mod, sites, nu, nd, fp32):
         S.scocg_destroy(h)
 
 
-# Hop lists of an even ring are read four entries at a time, of an odd one (or
-# an open chain's) singly; t, U, V and x are integers, so every form is exact.
+# A single apply: in compensated vectors the hop lists of an even ring are read
+# four entries at a time, of an odd one (or an open chain's) singly; complex128 reads
+# them singly.  t, U, V and x are integers, so every form is exact.
 @pytest.mark.parametrize("periodic", [True, False])
 @pytest.mark.parametrize("L,nu,nd", [(3, 1, 2), (5, 2, 3), (6, 3, 3), (7, 3, 4), (8, 4, 4), (9, 4, 3)])
 def test_ring_hop_lists(S, oracle_mod, L, nu, nd, periodic):
