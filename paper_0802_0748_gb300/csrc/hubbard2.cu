@@ -637,9 +637,12 @@ __device__ __forceinline__ double hop_sum_real(const double* amp, int S2, const 
     return hx;
 }
 
-__global__ void __launch_bounds__(kVecBlock) k_hub2_hx1(ApplyHubbard2<double> ap, int64_t nunits, const double* x,
-                                                        double* y, const double* xprev, const double* beta,
-                                                        double sigma, const int* skip) {
+// Five blocks per SM asked for: 42 registers, 5.64 ms per step of a ground state at 5
+// up / 5 down (0.916 at 4 up / 4 down).  Left to itself the compiler takes 32 and
+// schedules the two-word counts and the 32-bit division worse, 5.73 (0.923) ms.
+__global__ void __launch_bounds__(kVecBlock, 5) k_hub2_hx1(ApplyHubbard2<double> ap, int64_t nunits, const double* x,
+                                                           double* y, const double* xprev, const double* beta,
+                                                           double sigma, const int* skip) {
     if (skip && *skip) return;
     const int lane = threadIdx.x & 31;
     const int64_t w0 = (blockIdx.x * (int64_t)kVecBlock + threadIdx.x) >> 5;
