@@ -105,10 +105,10 @@ __device__ __forceinline__ void pk_acc_prod(float2& ah, float2& al, float2 xh, f
 // (ah, al) += v * (xh + xl) for an FP32 v, the apply's step: TwoProd, TwoSum and
 // one addition of both remainders to the low part.  (Folding the two exact
 // remainders (v xh - p) + (p - bb) into one fused operation v xh - bb takes 21
-// instead of 26 cycles of a scheduler's FP32 pipe per warp, 57.7 against 61 us
-// per iteration at 64^3 x 4, but rounds at the size of the sum where this step
-// rounds at the product's: the error of a 7-term sum grows by 2.5 %, of 28 terms
-// by 2.0 %.)
+// instead of 26 cycles of a scheduler's FP32 pipe per warp, and with the like form
+// of zx_minus 158 instead of 169 ms for 64^3 x 4 and 512 shifts, but rounds at the
+// size of the sum where this step rounds at the product's: the error of a 7-term
+// sum grows by 2.5 %, of 28 terms by 2.0 %.)
 __device__ __forceinline__ void pk_acc_fx2(float2& ah, float2& al, float2 v, float2 xh, float2 xl) {
     const float2 p = pk_mul(v, xh);
     const float2 e = pk_fma(v, xl, pk_fma(v, xh, pk_neg(p)));
