@@ -17,6 +17,8 @@ Ring ground states: odd rings, whose hop lists are read singly, and sectors with
 n_up != n_dn, whose diagonal table is not square; energies against dense
 eigenvalues.  A residual of 1e-10 leaves |dE| <= 1e-10.
 """
+import functools
+
 import numpy as np
 import pytest
 
@@ -57,6 +59,22 @@ def two_orbital(sites, fp32):
     return m
 
 
+Z = np.array([-3.0, 2.0, 7.0]) + 1.0j
+
+
+@functools.lru_cache(maxsize=None)
+def reference(oracle_mod, sites, nu, nd, fp32):
+    """Model, b and G of states 0, n / 2 and n - 1 at Z, [3][3]."""
+    from scipy.sparse import identity
+    from scipy.sparse.linalg import splu
+    m = two_orbital(sites, fp32)
+    H = sparse(oracle_mod.hubbard2_csr(m, nu, nd))
+    n = H.shape[0]
+    b = inputs.random_unit_complex(n, 11)
+    idx = [0, n // 2, n - 1]
+    return m, b, np.stack([splu((zk * identity(n) - H).tocsc()).solve(b)[idx] for zk in Z], axis=1)
+
+
 SECTORS = [(3, 2, 0), (3, 0, 2), (3, 2, 3), (3, 3, 4), (3, 6, 2), (4, 1, 3), (4, 3, 4), (4, 4, 3), (9, 2, 1), (9, 1, 2)]
 
 
@@ -64,20 +82,12 @@ SECTORS = [(3, 2, 0), (3, 0, 2), (3, 2, 3), (3, 3, 4), (3, 6, 2), (4, 1, 3), (4,
 @pytest.mark.parametrize("fp32", [True, False])
 @pytest.mark.parametrize("sites,nu,nd", SECTORS)
 def test_two_orbital_solve_rows(S, oracle_mod, sites, nu, nd, fp32, prec, tol, bound):
-    from scipy.sparse import identity
-    from scipy.sparse.linalg import splu
-    m = two_orbital(sites, fp32)
-    H = sparse(oracle_mod.hubbard2_csr(m, nu, nd))
-    n = H.shape[0]
-    b = inputs.random_unit_complex(n, 11)
-    z = np.array([-3.0, 2.0, 7.0]) + 1.0j
-    idx = [0, n // 2, n - 1]
-    want = np.stack([splu((zk * identity(n) - H).tocsc()).solve(b)[idx] for zk in z], axis=1)
+    m, b, want = reference(oracle_mod, sites, nu, nd, fp32)
     h = S.scocg_create_hubbard2(m, nu, nd, opts=S.SolveOptions(precision=prec))
     try:
         for grid in (0, 2):
             S.scocg_set_opts(h, S.SolveOptions(precision=prec, grid=grid))
-            G, info = S.scocg_solve(h, z, cuda(b), proj_idx=idx, tol=tol)
+            G, info = S.scocg_solve(h, Z, cuda(b), proj_idx=[0, b.size // 2, b.size - 1], tol=tol)
             assert info["status"] == 0 and info["iters"] <= 800
             assert np.max(np.abs(G.cpu().numpy()[0] - want)) <= bound, grid
     finally:
