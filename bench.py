@@ -90,7 +90,7 @@ from paper_0802_0748_gb300.inputs import ANDERSON64_BOUNDS as BOUNDS, BATCH32_BO
 # capture (dram__bytes_read.sum + dram__bytes_write.sum over a 60-iteration
 # launch on this workload, divided by 60; the command is in profiles/); valid
 # only for the kernel sources with this digest.
-TRAFFIC = {"digest": "5fb4adbb9d72631d", "df": (7.597751e9 + 8.653824e6) / 60}
+TRAFFIC = {"digest": "aafe46be1d49b814", "df": (7.599197e9 + 8.442880e6) / 60}
 
 
 # The sources of the persistent solve kernel and its launch (the kernel the
